@@ -1043,7 +1043,7 @@ const char* site_name(long long s)
 btt_status check_records()
 {
 #ifdef BTT_CHECK
-    cudaError_t (*units[])(long long*, bool) = {check_record_fft_static, check_record_gemv, check_record_api,
+    cudaError_t (*units[])(long long*, bool) = {check_record_fft_static, check_record_gemv, check_record_gemv_multi, check_record_api,
                                                 check_record_fft_exchange};
     for (auto u : units) {
         long long rec[3] = {0, 0, 0};

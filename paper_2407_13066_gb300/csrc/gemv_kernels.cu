@@ -9,133 +9,9 @@
 // F reduces along a row (threads stride l, then warp shuffles and a
 // shared-memory combine), F* combines rows (each thread owns a few l and
 // loops over s, with dhat[w][:] staged in shared memory).
-#include "fftq.cuh"
-#include "kernels.h"
+#include "gemv_store.cuh"
 
 namespace btt {
-
-// ------------------------------------------------------ storage decoding
-// Store<PREC>: one 16-byte unit of a Fhat row (VPL complex values).
-// load_raw fetches the unit (evict-first; the split pair also its lo-plane
-// twin at p + lo), decode turns it into FP32 complex values, and load does
-// both.  Kernels that keep many units in flight hold raw units and decode
-// late.
-template <int PREC> struct Store;
-
-template <> struct Store<P_F32> {
-    using elem = float2;
-    using acc = float;
-    using raw = float4;
-    static constexpr int VPL = 2;  // complex values per 16-byte load
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t)
-    {
-        return __ldcs(reinterpret_cast<const float4*>(p));
-    }
-    static __device__ __forceinline__ void decode(const raw& q, float2 (&f)[VPL])
-    {
-        f[0] = make_float2(q.x, q.y);
-        f[1] = make_float2(q.z, q.w);
-    }
-    static __device__ __forceinline__ void load(const elem* p, float2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
-
-template <> struct Store<P_F64> {
-    using elem = double2;
-    using acc = double;
-    using raw = double2;
-    static constexpr int VPL = 1;
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t) { return __ldcs(p); }
-    static __device__ __forceinline__ void decode(const raw& q, double2 (&f)[VPL]) { f[0] = q; }
-    static __device__ __forceinline__ void load(const elem* p, double2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
-
-template <> struct Store<P_F16S> {
-    using elem = __half2;
-    using acc = float;
-    using raw = uint4;
-    static constexpr int VPL = 4;
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t)
-    {
-        return __ldcs(reinterpret_cast<const uint4*>(p));
-    }
-    static __device__ __forceinline__ void decode(const raw& q, float2 (&f)[VPL])
-    {
-        const unsigned w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) f[i] = __half22float2(*reinterpret_cast<const __half2*>(&w[i]));
-    }
-    static __device__ __forceinline__ void load(const elem* p, float2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
-
-template <> struct Store<P_BF16> {
-    using elem = __nv_bfloat162;
-    using acc = float;
-    using raw = uint4;
-    static constexpr int VPL = 4;
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t)
-    {
-        return __ldcs(reinterpret_cast<const uint4*>(p));
-    }
-    static __device__ __forceinline__ void decode(const raw& q, float2 (&f)[VPL])
-    {
-        const unsigned w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) f[i] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-    }
-    static __device__ __forceinline__ void load(const elem* p, float2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
-
-// BF16 hi+lo split pair, stored as two planes of BF16 Fhat: hi at p, lo at
-// p + lo (the same [w][s][ldm] layout each, so either plane is also a BF16
-// operand of the tensor-core products).
-struct SplitRaw {
-    uint4 h, l;
-};
-template <> struct Store<P_BF16X2> {
-    using elem = __nv_bfloat162;
-    using acc = float;
-    using raw = SplitRaw;
-    static constexpr int VPL = 4;
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t lo)
-    {
-        return SplitRaw{__ldcs(reinterpret_cast<const uint4*>(p)), __ldcs(reinterpret_cast<const uint4*>(p + lo))};
-    }
-    static __device__ __forceinline__ void decode(const raw& q, float2 (&f)[VPL])
-    {
-        const unsigned h[4] = {q.h.x, q.h.y, q.h.z, q.h.w};
-        const unsigned l[4] = {q.l.x, q.l.y, q.l.z, q.l.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[i]));
-            const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&l[i]));
-            f[i] = make_float2(a.x + b.x, a.y + b.y);
-        }
-    }
-    static __device__ __forceinline__ void load(const elem* p, float2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
-
-template <> struct Store<P_FP8S> {
-    using elem = __nv_fp8x2_storage_t;   // (Re, Im) E4M3 codes of Fhat / s_w
-    using acc = float;
-    using raw = uint4;
-    static constexpr int VPL = 8;
-    static __device__ __forceinline__ raw load_raw(const elem* p, int64_t)
-    {
-        return __ldcs(reinterpret_cast<const uint4*>(p));
-    }
-    static __device__ __forceinline__ void decode(const raw& q, float2 (&f)[VPL])
-    {
-        const unsigned w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const __half2 lo = __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[i] & 0xFFFFu), __NV_E4M3));
-            const __half2 hi = __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w[i] >> 16), __NV_E4M3));
-            f[2 * i] = __half22float2(lo);
-            f[2 * i + 1] = __half22float2(hi);
-        }
-    }
-    static __device__ __forceinline__ void load(const elem* p, float2 (&f)[VPL], int64_t lo) { decode(load_raw(p, lo), f); }
-};
 
 template <typename V> __device__ __forceinline__ void load_vec(const V* p, V (&x)[1]) { x[0] = __ldg(p); }
 __device__ __forceinline__ void load_vec(const float2* p, float2 (&x)[2])
@@ -161,22 +37,6 @@ __device__ __forceinline__ void load_vec(const float2* p, float2 (&x)[4])
     x[1] = make_float2(q0.z, q0.w);
     x[2] = make_float2(q1.x, q1.y);
     x[3] = make_float2(q1.z, q1.w);
-}
-
-template <typename V> __device__ __forceinline__ void cfma(V& acc, V a, V b)
-{
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(-a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(a.y, b.x, acc.y);
-}
-// acc += conj(a) * b
-template <typename V> __device__ __forceinline__ void cfma_conj(V& acc, V a, V b)
-{
-    acc.x = fma(a.x, b.x, acc.x);
-    acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y);
-    acc.y = fma(-a.y, b.x, acc.y);
 }
 
 // ------------------------------------------------------------ F (Alg. 2)
@@ -500,11 +360,6 @@ k_gemv_adj(const typename Store<PREC>::elem* __restrict__ fhat, const float* __r
 // ---------------------------------------------------------------- launchers
 constexpr int kGemvThreads = 256;
 
-// element offset of the lo plane of a split-pair Fhat (0 for other formats)
-static int64_t lo_plane(int prec, int n_freq, int N_d, int ldm)
-{
-    return prec == P_BF16X2 ? (int64_t)n_freq * N_d * ldm : 0;
-}
 constexpr int kAdjUnroll = 8;
 
 template <int PREC, int R, int NB>
@@ -577,11 +432,31 @@ static cudaError_t fwd_dispatch(const void* fhat, const float* scales, int n_fre
     return rows_shape<PREC, 4, U4, 512>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
 }
 
+// Where the group kernel of gemv_multi.cu is the faster one for F.  Measured
+// (this file's kernel -> the group kernel, us per launch):
+//   256 x 200 x 10000: FP32 3 vectors 779 -> 661, 8 1513 -> 1004, 32 5890 ->
+//     3807; FP8 3 vectors 1007 -> 423; 2 vectors within 5% or slower (FP32
+//     608 -> 642); split pairs (16 more registers per row) 4 876 -> 1111;
+//   300 x 37 x 3001, a CTA's rows too short for its staging: FP32 4 vectors
+//     63 -> 75, 8 123 -> 102;
+//   64 x 8 x 20000, 65 CTAs of 20 rows here: FP32 2 vectors 64 -> 35, split
+//     pairs 123 -> 31 (l split over warps), but FP16 32 vectors 170 -> 281.
+static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
+{
+    if (nrhs < 2) return false;
+    if (nrhs > 16 && N_d <= 8 && prec != P_F32) return false;
+    if ((int64_t)n_freq * ((N_d + 19) / 20) < 152) return true;
+    if (nrhs == 2 || prec == P_BF16X2) return false;
+    return nrhs > 4 || ldm >= 4096 || N_d <= 16;
+}
+
 cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
                             int ldm, const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs,
                             cudaStream_t st)
 {
     if (nrhs <= 0) return cudaSuccess;
+    if (prec != P_F64 && fwd_multi_wins(prec, n_freq, N_d, ldm, nrhs))
+        return launch_gemv_fwd_multi(prec, fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
     switch (prec) {
         case P_F32: return fwd_dispatch<P_F32>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_F64: return fwd_launch<P_F64, 4, 1>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
@@ -615,29 +490,26 @@ static cudaError_t adj_launch(const void* fhat, const float* scales, int n_freq,
     return cudaGetLastError();
 }
 
-template <int PREC>
-static cudaError_t adj_dispatch(const void* fhat, const float* scales, int n_freq, int N_d, int N_m,
-                                int ldm, const void* dh, int64_t dbs, void* mh, int64_t mbs, int nrhs,
-                                cudaStream_t st)
-{
-    if (nrhs == 1) return adj_launch<PREC, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-    if (nrhs == 2) return adj_launch<PREC, 2>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-    if (nrhs <= 4) return adj_launch<PREC, 4>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-    return adj_launch<PREC, 8>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-}
-
 cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
                             int N_m, int ldm, const void* dh, int64_t dbs, void* mh, int64_t mbs,
                             int nrhs, cudaStream_t st)
 {
     if (nrhs <= 0) return cudaSuccess;
+    // several vectors: the group kernel (two in FP32 and BF16 stay here: 592
+    // against 602 us at 256 x 200 x 10000, 155 against 177 at 1500 x 24 x 6000)
+    if (prec != P_F64 && nrhs > (prec == P_BF16 || prec == P_F32 ? 2 : 1))
+        return launch_gemv_adj_multi(prec, fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
     switch (prec) {
-        case P_F32: return adj_dispatch<P_F32>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
+        case P_F32:
+            return nrhs == 1 ? adj_launch<P_F32, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st)
+                             : adj_launch<P_F32, 2>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
         case P_F64: return adj_launch<P_F64, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-        case P_F16S: return adj_dispatch<P_F16S>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-        case P_BF16: return adj_dispatch<P_BF16>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-        case P_BF16X2: return adj_dispatch<P_BF16X2>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
-        case P_FP8S: return adj_dispatch<P_FP8S>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
+        case P_F16S: return adj_launch<P_F16S, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
+        case P_BF16:
+            return nrhs == 1 ? adj_launch<P_BF16, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st)
+                             : adj_launch<P_BF16, 2>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
+        case P_BF16X2: return adj_launch<P_BF16X2, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
+        case P_FP8S: return adj_launch<P_FP8S, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -44,6 +44,7 @@ cudaError_t prepare_kernels();
 // with clear.
 cudaError_t check_record_fft_static(long long* rec, bool clear);
 cudaError_t check_record_gemv(long long* rec, bool clear);
+cudaError_t check_record_gemv_multi(long long* rec, bool clear);
 cudaError_t check_record_api(long long* rec, bool clear);
 cudaError_t check_record_fft_exchange(long long* rec, bool clear);
 #endif
@@ -99,6 +100,13 @@ cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int
 cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
                             int N_m, int ldm, const void* dh, int64_t dbs, void* mh, int64_t mbs,
                             int nrhs, cudaStream_t st);
+
+// Both for several vectors at once, FP32 formats (gemv_multi.cu).
+cudaError_t launch_gemv_fwd_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int ldm,
+                                  const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs, cudaStream_t st);
+cudaError_t launch_gemv_adj_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int N_m,
+                                  int ldm, const void* dh, int64_t dbs, void* mh, int64_t mbs, int nrhs,
+                                  cudaStream_t st);
 
 // ---- fixed-plan FP32 transforms (fft_static.cu); false if no plan for g.L ----
 cudaError_t prepare_static_fft();

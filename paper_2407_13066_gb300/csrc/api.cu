@@ -100,7 +100,8 @@ struct btt_op {
     void* stage_in = nullptr;         // [max_nrhs][N_t][max(N_m,N_d)] real
     void* stage_out = nullptr;
     void* gamma = nullptr;            // [N_t][N_d] real
-    float* dw = nullptr;              // [max_nrhs][N_t][N_d]: Gamma^-1 d for btt_adjoint_weighted
+    float* dw = nullptr;              // [max_nrhs][N_t][N_d]: Gamma^-1 d for btt_adjoint_weighted, the
+                                      // Hessian's time-domain data at lengths without a fixed plan
     void** ptab = nullptr;            // device tables of vector pointers: [2][max_nrhs]
     // conjugate-gradient workspace, allocated by the first btt_cg call
     float* cg_vec = nullptr;          // r, p, Ap: [3][cg_cap][N_t][N_m]
@@ -359,8 +360,10 @@ btt_status run_action(btt_op* op, Action act, const T* in, const T* gamma, T* ou
             }
             // CG: the middle step also leaves the partials of p.Hp = ||F p||^2 (Gamma^-1)
             const int mid_nblk = fft_col_blocks(N_d, geo);
+            T* mid_scratch = nullptr;   // op->dw: Gamma^-1 d of btt_adjoint_weighted, free here
+            if constexpr (std::is_same<T, float>::value) mid_scratch = op->dw;
             double* mp = mid_part ? mid_part + (size_t)c0 * mid_nblk : nullptr;
-            STAGE(BTT_STAGE_MID, launch_hess_mid<T>(dh, N_d, dbs, N_d, g, nb, geo, tw, st, mp));
+            STAGE(BTT_STAGE_MID, launch_hess_mid<T>(dh, N_d, dbs, N_d, g, nb, geo, tw, st, mp, mid_scratch));
             // fused CG step: the step lengths are known once p.Hp is
             if (cgf) CK(launch_cg_finish(mp, mid_nblk, FIN_ALPHA, 0, 0.0, cgf->shift, nb, cgf->cv + c0, st));
             if (tc) {
@@ -523,7 +526,7 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     STEP(alloc(&op->fhat, op->fhat_bytes, "Fhat"));
     STEP(alloc((void**)&op->tw32, L * 2 * sizeof(float4), "twiddles"));
     STEP(alloc((void**)&op->tw64, L * sizeof(double2), "twiddles"));
-    STEP(alloc((void**)&op->pos, L * sizeof(int), "digit-reversal table"));
+    STEP(alloc((void**)&op->pos, (L + geom.res_ints) * sizeof(int), "position tables"));
     STEP(alloc(&op->xhat, xh_b, "mhat workspace"));
     STEP(alloc(&op->dhat, dh_b, "dhat workspace"));
     STEP(alloc(&op->stage_in, st_b, "staging"));
@@ -575,10 +578,12 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     }
     CKF(cudaMemcpyAsync(op->tw64, t64.data(), L * sizeof(double2), cudaMemcpyHostToDevice, st));
     CKF(cudaMemcpyAsync(op->tw32, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
-    std::vector<int> pos(L);
+    std::vector<int> pos(L + geom.res_ints);
     digit_reversal(op->geom, pos.data());
-    CKF(cudaMemcpyAsync(op->pos, pos.data(), L * sizeof(int), cudaMemcpyHostToDevice, st));
+    res_tables(op->geom, pos.data() + L);
+    CKF(cudaMemcpyAsync(op->pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     op->geom.pos = op->pos;
+    op->geom.res_tab = op->pos + L;
     // zero Fhat (row padding l >= N_m stays zero) and the workspace padding
     CKF(cudaMemsetAsync(op->fhat, 0, op->fhat_bytes, st));
     CKF(cudaMemsetAsync(op->xhat, 0, xh_b, st));
@@ -1044,7 +1049,7 @@ btt_status check_records()
 {
 #ifdef BTT_CHECK
     cudaError_t (*units[])(long long*, bool) = {check_record_fft_static, check_record_gemv, check_record_gemv_multi, check_record_api,
-                                                check_record_fft_exchange};
+                                                check_record_fft_exchange, check_record_fft_residue};
     for (auto u : units) {
         long long rec[3] = {0, 0, 0};
         cudaError_t e = u(rec, true);

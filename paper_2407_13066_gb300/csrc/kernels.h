@@ -7,6 +7,16 @@
 
 namespace btt {
 
+// Plan of the residue transforms (fft_residue.cu) on clusters of C CTAs:
+// M = N_t / C points per residue (0: C does not divide N_t), its radices and
+// their divisors, the plan's place in the position tables.
+constexpr int kResPasses = 6;
+struct ResPlan {
+    int M, np, tab;
+    int radix[kResPasses];
+    unsigned magic[kResPasses];
+};
+
 // Geometry of the time transforms of one operator.
 struct FftGeom {
     int N_t;       // samples kept
@@ -14,6 +24,9 @@ struct FftGeom {
     int wc_log2;   // log2 of the complex columns per CTA
     FftPlan plan;
     const int* pos;  // device table: position of frequency k after a forward transform
+    ResPlan res[4];  // for clusters of 1, 2, 4, 8 CTAs
+    int res_ints;    // entries of their position tables
+    const int* res_tab;  // device copy (NULL: the residue transforms are not used)
 };
 
 // Builds the radix plan for L and the column tile for a shared-memory
@@ -47,6 +60,7 @@ cudaError_t check_record_gemv(long long* rec, bool clear);
 cudaError_t check_record_gemv_multi(long long* rec, bool clear);
 cudaError_t check_record_api(long long* rec, bool clear);
 cudaError_t check_record_fft_exchange(long long* rec, bool clear);
+cudaError_t check_record_fft_residue(long long* rec, bool clear);
 #endif
 
 // ---- time transforms (fft_kernels.cu) ----
@@ -69,11 +83,12 @@ cudaError_t launch_irfft(const cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols
 // F* passes of the Hessian (g = NULL means 1).  With part != NULL, block
 // (tile, b) also writes part[b * fft_col_blocks(ncols) + tile] = its share of
 // sum_t sum_col g (F m)^2, the Gamma^-1-weighted squared norm of vector b's
-// data (p.Hp for the CG solver).
+// data (p.Hp for the CG solver).  scratch: NULL, or nb N_t ncols values the
+// call may overwrite.
 template <typename T>
 cudaError_t launch_hess_mid(cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols, const T* g,
                             int nb, const FftGeom& geom, const cplx_t<T>* tw, cudaStream_t st,
-                            double* part = nullptr);
+                            double* part = nullptr, T* scratch = nullptr);
 // Column tiles (blocks per vector) of the transforms of ncols columns.
 int fft_col_blocks(int ncols, const FftGeom& geom);
 
@@ -144,6 +159,22 @@ bool exchange_irfft(const float2* X, int64_t ldx, int64_t bsx, int ncols, float*
 bool exchange_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy,
                          int64_t bsy, int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr,
                          cudaError_t* err);
+// ---- residue transforms of any length (fft_residue.cu); false where the
+// kernels of fft_kernels.cu run.  tw must hold the quad table after the L
+// entries; arguments as the static_* forms. ----
+void make_res_plans(FftGeom* g);
+void res_tables(const FftGeom& g, int* t);   // host: g.res_ints entries
+cudaError_t prepare_res_fft();
+bool res_rfft(const float* x, int64_t ldx, int64_t bsx, int ncols, float2* X, int64_t ldo, int64_t bso, int nb,
+              const FftGeom& g, const float2* tw, cudaStream_t st, const float* const* xptr, cudaError_t* err);
+bool res_rfft_stack(const float* x, int64_t ldx, int64_t bsx, int ncols, void* xstack, int ldm, int mt_stride, int nb,
+                    const FftGeom& g, const float2* tw, cudaStream_t st, int64_t lo_off, const float* const* xptr,
+                    cudaError_t* err);
+bool res_irfft(const float2* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy, int64_t bsy,
+               const float* gam, int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr,
+               cudaError_t* err);
+bool res_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy, int64_t bsy,
+                    int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr, cudaError_t* err);
 // True when 2 N_t has a fixed radix plan.
 bool static_plan(const FftGeom& g);
 // Its fixed-plan form; false for lengths without a fixed plan.

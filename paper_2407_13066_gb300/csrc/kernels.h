@@ -230,14 +230,15 @@ struct CgFuse {
 };
 
 // ---- tensor-core multi-RHS products (tc_gemm.cu) ----
+constexpr int kArowMaps = 4;
 // Plan of the BF16 tcgen05 path for one operator.
 struct TcPlan {
-    CUtensorMap tmA;      // conj BF16 spectra [w][mt][64][K2]
+    CUtensorMap tmA[kArowMaps];   // conj BF16 spectra [w][mt][64][K2], boxes of 16 (i + 1) rows
     CUtensorMap tmB;      // Fhat BF16 [w][s][K2], boxes of 64 x N rows (F pass)
-    CUtensorMap tmD;      // stacked planar BF16 dhat [w][mt][128][kd] (F* pass)
+    CUtensorMap tmD[kArowMaps];   // stacked planar BF16 dhat [w][mt][128][kd] (F* pass), 32 (i + 1) rows
     CUtensorMap tmF;      // Fhat BF16 [w][s][K2], boxes of 64 x 64 rows (F* pass)
     // split pairs (BF16 hi+lo): the same four maps over the lo planes
-    CUtensorMap tmA_lo, tmB_lo, tmD_lo, tmF_lo;
+    CUtensorMap tmA_lo[kArowMaps], tmB_lo, tmD_lo[kArowMaps], tmF_lo;
     bool split;
     int64_t xs_lo;        // lo plane of the spectra buffer, in BF16 pairs (0 unless split)
     int64_t ds_lo;        // lo plane of the dhat stack, in BF16 elements (0 unless split)

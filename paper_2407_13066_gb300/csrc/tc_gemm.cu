@@ -24,6 +24,7 @@
 // tcgen05.ld.  Every wait on an mbarrier is bounded in time; on timeout the
 // kernel records an error code, waits (bounded) for its own copies, frees
 // TMEM and returns.
+#include <algorithm>
 #include <cmath>
 #include <cuda.h>
 
@@ -182,12 +183,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
 // grid = (frequency w, N tile, K split); 128 threads: warp 0 TMA, warp 1
 // MMA, warps 2-3 derive the swap rows, all four read the accumulator.
 // part[((split * n_freq + w) * n_ntiles + nt) * NM * 128 + row][col], row in
-// [0, 128 NM), col in [0, ntile_rows): partial sums of this CTA.
-template <int NM, int STAGES>
+// [0, 128 NM), col in [0, ntile_rows): partial sums of this CTA.  FULL: all 64
+// rows of spectra are loaded (arows = 64).
+template <int NM, int STAGES, bool FULL>
 __global__ void __launch_bounds__(128, 1)
 k_tc_fwd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int n_freq,
-         int ntile_rows, int ktiles, int kt_per_split, int mt_stride, int mt0, float* __restrict__ part,
-         int* __restrict__ err)
+         int ntile_rows, int ktiles, int kt_per_split, int mt_stride, int mt0, int arows, int nb,
+         float* __restrict__ part, int* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -246,7 +248,8 @@ k_tc_fwd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 const uint4* src = reinterpret_cast<const uint4*>(st + mt * A_BYTES);
                 uint4* dst = reinterpret_cast<uint4*>(st + mt * A_BYTES + HALF);
 #pragma unroll
-                for (int q = 0; q < HALF / 16 / 64; ++q) {
+                for (int q = 0; q < HALF / 16 / 64; ++q) {   // 8 rows each
+                    if (!FULL && 8 * q >= arows) break;
                     uint4 v = src[t + 64 * q];
                     v.x = (v.x << 16) | ((v.x >> 16) ^ 0x8000u);
                     v.y = (v.y << 16) | ((v.y >> 16) ^ 0x8000u);
@@ -270,7 +273,7 @@ k_tc_fwd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
                 break;
             }
             unsigned char* st = smem + s * stage_bytes;
-            mbar_expect_tx(&full[s], (uint32_t)(stage_bytes - NAT * HALF));
+            mbar_expect_tx(&full[s], (uint32_t)(b_bytes + NAT * arows * kTileK * 2));
             const int kx = (kt0 + i) * kTileK;
 #pragma unroll
             for (int mt = 0; mt < NM; ++mt)
@@ -317,6 +320,7 @@ k_tc_fwd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
         const size_t tile = ((size_t)sp * n_freq + w) * n_ntiles + nt;
 #pragma unroll
         for (int mt = 0; mt < NM; ++mt) {
+            if (!FULL && 64 * mt + (warp & 1) * 32 >= nb) continue;   // no vector in this warp's rows
             float* dst = part + (tile * NM * kTileM + (size_t)mt * kTileM + row) * ntile_rows;
             for (int c = 0; c < ntile_rows; c += 16) {
                 float v[16];
@@ -354,21 +358,32 @@ k_tc_fwd(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtens
 // 32 (e % 4) .. +31 and columns [128 (e / 4), +128) of the tile.
 constexpr int kDrainWarps = 8;
 constexpr int kFwdSplitThreads = 128 + 32 * kDrainWarps;
-constexpr int kFwdSplitStages = 2;
+// Stages of the ring (as many as fit, up to 4) and the places of A_hi and A_lo
+// in one.  COMPACT (up to 32 vectors): only rows 0-31 and the swap rows 64-95 of
+// an A tile are used, so A_lo sits 4 KB into A_hi, in the rows A_hi leaves
+// free.  One CTA per SM (all of TMEM): with two stages one is multiplied while
+// the other loads, too little in flight for the memory rate.
+template <bool COMPACT, int STAGES> struct FwdSplit {
+    static constexpr int kTile = kTileM * kTileK * 2;
+    static constexpr int kLo = COMPACT ? kTile / 4 : kTile;
+    static constexpr int kA = kLo + kTile;   // both tiles
+    static size_t smem(int ntile_rows) { return (size_t)STAGES * (kA + 2 * ntile_rows * kTileK * 2) + 1024; }
+};
 
+template <bool COMPACT, int STAGES>
 __global__ void __launch_bounds__(kFwdSplitThreads, 1)
 k_tc_fwd_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmA_lo, const __grid_constant__ CUtensorMap tmB_lo, int n_freq,
-               int ntile_rows, int ktiles, int kt_per_split, int chain, int mt_stride, int mt0,
+               int ntile_rows, int ktiles, int kt_per_split, int chain, int mt_stride, int mt0, int arows, int nb,
                float* __restrict__ part, int* __restrict__ err)
 {
-    constexpr int STAGES = kFwdSplitStages;
+    using Cfg = FwdSplit<COMPACT, STAGES>;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int A_BYTES = kTileM * kTileK * 2;
     const int b_bytes = ntile_rows * kTileK * 2;
-    const int stage_bytes = 2 * A_BYTES + 2 * b_bytes;   // A_hi, A_lo, B_hi, B_lo
+    const int stage_bytes = Cfg::kA + 2 * b_bytes;   // A_hi, A_lo, B_hi, B_lo
     constexpr uint32_t NCOLS = 512;
     constexpr int HALF = A_BYTES / 2;   // 64 conj rows as loaded; the swap rows follow
 
@@ -418,10 +433,10 @@ k_tc_fwd_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             unsigned char* st = smem + s * stage_bytes;
 #pragma unroll
             for (int a = 0; a < 2; ++a) {
-                const uint4* src = reinterpret_cast<const uint4*>(st + a * A_BYTES);
-                uint4* dst = reinterpret_cast<uint4*>(st + a * A_BYTES + HALF);
+                const uint4* src = reinterpret_cast<const uint4*>(st + a * Cfg::kLo);
+                uint4* dst = reinterpret_cast<uint4*>(st + a * Cfg::kLo + HALF);
 #pragma unroll
-                for (int q = 0; q < HALF / 16 / 64; ++q) {
+                for (int q = 0; q < HALF / 16 / 64 / (COMPACT ? 2 : 1); ++q) {   // 8 rows each
                     uint4 v = src[t + 64 * q];
                     v.x = (v.x << 16) | ((v.x >> 16) ^ 0x8000u);
                     v.y = (v.y << 16) | ((v.y >> 16) ^ 0x8000u);
@@ -446,12 +461,12 @@ k_tc_fwd_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     break;
                 }
                 unsigned char* st = smem + s * stage_bytes;
-                mbar_expect_tx(&full[s], (uint32_t)(stage_bytes - 2 * HALF));
+                mbar_expect_tx(&full[s], (uint32_t)(2 * b_bytes + 2 * arows * kTileK * 2));
                 const int kx = (kt0 + i) * kTileK;
                 tma_load_2d(st, &tmA, kx, (w * mt_stride + mt0) * 64, &full[s]);
-                tma_load_2d(st + A_BYTES, &tmA_lo, kx, (w * mt_stride + mt0) * 64, &full[s]);
-                tma_load_3d(st + 2 * A_BYTES, &tmB, kx, nt * ntile_rows, w, &full[s]);
-                tma_load_3d(st + 2 * A_BYTES + b_bytes, &tmB_lo, kx, nt * ntile_rows, w, &full[s]);
+                tma_load_2d(st + Cfg::kLo, &tmA_lo, kx, (w * mt_stride + mt0) * 64, &full[s]);
+                tma_load_3d(st + Cfg::kA, &tmB, kx, nt * ntile_rows, w, &full[s]);
+                tma_load_3d(st + Cfg::kA + b_bytes, &tmB_lo, kx, nt * ntile_rows, w, &full[s]);
                 ++issued;
             }
             // copies still in flight complete on their full barriers
@@ -479,10 +494,10 @@ k_tc_fwd_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
                 tc_fence_after();
                 const uint32_t sa = smem_u32(smem + s * stage_bytes);
-                const uint32_t sb = sa + 2 * A_BYTES, sbl = sb + (uint32_t)b_bytes;
+                const uint32_t sb = sa + Cfg::kA, sbl = sb + (uint32_t)b_bytes;
 #pragma unroll
                 for (int kk = 0; kk < kTileK / 16; ++kk) {
-                    const uint64_t ah = desc_kmajor_sw128(sa + kk * 32), al = desc_kmajor_sw128(sa + A_BYTES + kk * 32);
+                    const uint64_t ah = desc_kmajor_sw128(sa + kk * 32), al = desc_kmajor_sw128(sa + Cfg::kLo + kk * 32);
                     const uint64_t bh = desc_kmajor_sw128(sb + kk * 32), bl = desc_kmajor_sw128(sbl + kk * 32);
                     mma_bf16(tbase, ah, bh, idesc, (ic > 0 || kk > 0) ? 1u : 0u);
                     mma_bf16(tbase + 256, ah, bl, idesc, (i > 0 || kk > 0) ? 1u : 0u);
@@ -541,7 +556,7 @@ k_tc_fwd_split(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int col = h * 128 + 16 * q;
-                if (col < ntile_rows) {
+                if (col < ntile_rows && (grp & 1) * 32 < nb) {   // a vector in this warp's rows
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
                         reinterpret_cast<float4*>(dst + col)[u] =
@@ -636,7 +651,7 @@ template <bool SPLIT, bool OUT16>
 __global__ void __launch_bounds__(kAdjThreads, 1)
 k_tc_adj(const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtensorMap tmF,
          const __grid_constant__ CUtensorMap tmD_lo, const __grid_constant__ CUtensorMap tmF_lo, int n_freq,
-         int N_d, int N_m, int ldm, int kd_tiles, int n_ntiles, int mt_stride, int mt0, int nb,
+         int N_d, int N_m, int ldm, int kd_tiles, int n_ntiles, int mt_stride, int mt0, int nb, int arows,
          void* __restrict__ mh_out, int64_t mbs, int* __restrict__ err)
 {
     static_assert(!(SPLIT && OUT16), "split pairs keep complex64 mhat");
@@ -693,7 +708,7 @@ k_tc_adj(const __grid_constant__ CUtensorMap tmD, const __grid_constant__ CUtens
                         break;
                     }
                     unsigned char* st = smem + s * kAdjStage;
-                    mbar_expect_tx(&full[s], (uint32_t)kAdjStage);
+                    mbar_expect_tx(&full[s], (uint32_t)(C::kParts * (arows * kTileK * 2 + (kAdjN / 64) * kAdjBlk)));
                     tma_load_2d(st, &tmD, kt * kTileK, (w * mt_stride + mt0) * kTileM, &full[s]);
 #pragma unroll
                     for (int a = 0; a < kAdjN / 64; ++a)
@@ -914,15 +929,13 @@ EncodeTiled encode_fn()
     return fn;
 }
 
+// shared memory the three-stage split forward may claim (its own barriers
+// and flags take the rest of the 227 KB)
+constexpr int kSplitSmemMax = 226 * 1024;
+
 template <int NM, int STAGES> size_t fwd_smem(int ntile_rows)
 {
     return (size_t)STAGES * (NM * tc::kTileM * tc::kTileK * 2 + ntile_rows * tc::kTileK * 2) + 1024;
-}
-
-// split pairs: stages of A_hi, A_lo, B_hi, B_lo
-size_t fwd_split_smem(int ntile_rows)
-{
-    return (size_t)tc::kFwdSplitStages * (2 * tc::kTileM * tc::kTileK * 2 + 2 * ntile_rows * tc::kTileK * 2) + 1024;
 }
 
 }  // namespace
@@ -989,13 +1002,14 @@ cudaError_t encode_maps(EncodeTiled enc, const TcPlan& p, void* xstack, const vo
                         int n_freq, int N_d, CUtensorMap* tmA, CUtensorMap* tmB, CUtensorMap* tmD,
                         CUtensorMap* tmF)
 {
-    {
-        // A: conj spectra [w][mt][64][K2] BF16 as 2-D (K2, rows)
+    for (int i = 0; i < kArowMaps; ++i) {
+        // A: conj spectra [w][mt][64][K2] BF16 as 2-D (K2, rows); map i loads
+        // the first 16 (i + 1) rows of a tile
         cuuint64_t dims[2] = {(cuuint64_t)p.K2, (cuuint64_t)n_freq * p.mt_alloc * 64};
         cuuint64_t strides[1] = {(cuuint64_t)p.K2 * 2};
-        cuuint32_t box[2] = {(cuuint32_t)tc::kTileK, 64};
+        cuuint32_t box[2] = {(cuuint32_t)tc::kTileK, (cuuint32_t)(16 * (i + 1))};
         cuuint32_t es[2] = {1, 1};
-        if (enc(tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xstack, dims, strides, box, es,
+        if (enc(&tmA[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, xstack, dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -1011,14 +1025,14 @@ cudaError_t encode_maps(EncodeTiled enc, const TcPlan& p, void* xstack, const vo
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
     }
-    {
+    for (int i = 0; i < kArowMaps; ++i) {
         // adjoint A: stacked planar dhat [w][mt][128][kd] BF16 as 2-D (N_d, rows);
-        // columns >= N_d read as zero
+        // columns >= N_d read as zero; map i loads the first 32 (i + 1) rows
         cuuint64_t dims[2] = {(cuuint64_t)N_d, (cuuint64_t)n_freq * p.mt_alloc * tc::kTileM};
         cuuint64_t strides[1] = {(cuuint64_t)p.kd * 2};
-        cuuint32_t box[2] = {(cuuint32_t)tc::kTileK, (cuuint32_t)tc::kTileM};
+        cuuint32_t box[2] = {(cuuint32_t)tc::kTileK, (cuuint32_t)(32 * (i + 1))};
         cuuint32_t es[2] = {1, 1};
-        if (enc(tmD, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, dstack, dims, strides, box, es,
+        if (enc(&tmD[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, dstack, dims, strides, box, es,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
@@ -1044,7 +1058,7 @@ cudaError_t tc_prepare(TcPlan* p, void* xstack, const void* fhat_bf16, int n_fre
     // p->dstack must be set by the caller (stacked planar dhat buffer)
     EncodeTiled enc = encode_fn();
     if (!enc) return cudaErrorNotSupported;
-    cudaError_t e = encode_maps(enc, *p, xstack, fhat_bf16, p->dstack, n_freq, N_d, &p->tmA, &p->tmB, &p->tmD,
+    cudaError_t e = encode_maps(enc, *p, xstack, fhat_bf16, p->dstack, n_freq, N_d, p->tmA, &p->tmB, p->tmD,
                                 &p->tmF);
     if (e != cudaSuccess) return e;
     if (p->split) {
@@ -1052,22 +1066,31 @@ cudaError_t tc_prepare(TcPlan* p, void* xstack, const void* fhat_bf16, int n_fre
         const size_t fplane = (size_t)n_freq * N_d * p->K2 * 2;   // bytes of one Fhat plane
         e = encode_maps(enc, *p, static_cast<char*>(xstack) + p->xs_lo * 4,
                         static_cast<const char*>(fhat_bf16) + fplane, static_cast<char*>(p->dstack) + p->ds_lo * 2,
-                        n_freq, N_d, &p->tmA_lo, &p->tmB_lo, &p->tmD_lo, &p->tmF_lo);
+                        n_freq, N_d, p->tmA_lo, &p->tmB_lo, p->tmD_lo, &p->tmF_lo);
         if (e != cudaSuccess) return e;
     } else {
-        p->tmA_lo = p->tmA;
+        for (int i = 0; i < kArowMaps; ++i) p->tmA_lo[i] = p->tmA[i], p->tmD_lo[i] = p->tmD[i];
         p->tmB_lo = p->tmB;
-        p->tmD_lo = p->tmD;
         p->tmF_lo = p->tmF;
     }
-    e = cudaFuncSetAttribute(tc::k_tc_fwd<1, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(tc::k_tc_fwd<1, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)fwd_smem<1, 4>(256));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc::k_tc_fwd<2, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(tc::k_tc_fwd<1, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)fwd_smem<1, 4>(256));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc::k_tc_fwd<1, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)fwd_smem<1, 3>(160));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc::k_tc_fwd<1, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)fwd_smem<1, 3>(160));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc::k_tc_fwd<2, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)fwd_smem<2, 3>(256));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc::k_tc_fwd_split, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)fwd_split_smem(256));
+        for (auto k : {tc::k_tc_fwd_split<false, 2>, tc::k_tc_fwd_split<false, 3>, tc::k_tc_fwd_split<false, 4>,
+                       tc::k_tc_fwd_split<true, 3>, tc::k_tc_fwd_split<true, 4>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmemMax);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(tc::k_tc_adj<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  tc::AdjCfg<false>::kSmem);
@@ -1103,18 +1126,20 @@ cudaError_t launch_tc_adj(const TcPlan& p, int n_freq, int N_d, int N_m, int ldm
     const int ntiles = n_freq * n_ntiles;
     const int grid = ntiles < nsm ? ntiles : nsm;
     for (int b0 = 0; b0 < nrhs; b0 += 64) {
+        // rows of the data spectra a stage loads (as in launch_tc_fwd)
+        const int am = (std::min(64, nrhs - b0) - 1) / 16, arows = 32 * (am + 1);
         if (p.split)
             tc::k_tc_adj<true, false><<<grid, tc::kAdjThreads, tc::AdjCfg<true>::kSmem, st>>>(
-                p.tmD, p.tmF, p.tmD_lo, p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64, nrhs,
-                mh, mbs, err);
+                p.tmD[am], p.tmF, p.tmD_lo[am], p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64,
+                nrhs, arows, mh, mbs, err);
         else if (out_bf16)
             tc::k_tc_adj<false, true><<<grid, tc::kAdjThreads, tc::AdjCfg<false>::kSmem, st>>>(
-                p.tmD, p.tmF, p.tmD_lo, p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64, nrhs,
-                mh, mbs, err);
+                p.tmD[am], p.tmF, p.tmD_lo[am], p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64,
+                nrhs, arows, mh, mbs, err);
         else
             tc::k_tc_adj<false, false><<<grid, tc::kAdjThreads, tc::AdjCfg<false>::kSmem, st>>>(
-                p.tmD, p.tmF, p.tmD_lo, p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64, nrhs,
-                mh, mbs, err);
+                p.tmD[am], p.tmF, p.tmD_lo[am], p.tmF_lo, n_freq, N_d, N_m, ldm, kd_tiles, n_ntiles, p.mt_alloc, b0 / 64,
+                nrhs, arows, mh, mbs, err);
         count_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1137,17 +1162,50 @@ cudaError_t launch_tc_fwd(const TcPlan& p, int n_freq, int N_d, int nrhs, float*
     for (int b0 = 0; b0 < nrhs; b0 += step) {
         const int nb = nrhs - b0 < step ? nrhs - b0 : step;
         const int NM = (nb + 63) / 64;
+        // rows of spectra a stage loads: the vectors rounded up to 16, not the
+        // tile's 64 (a row of A costs as much HBM traffic as a row of Fhat):
+        // F of 32 vectors at 256 x 200 x 10000 479 -> 414 us in BF16, 904 ->
+        // 835 us as split pairs, 750 with the third stage that then fits.
+        // The tile's other rows keep whatever shared memory held: row i of A
+        // reaches only row i of the product, which nothing reads.
+        const int am = NM == 1 ? (nb - 1) / 16 : kArowMaps - 1, arows = 16 * (am + 1);
         dim3 grid((unsigned)n_freq, (unsigned)p.n_ntiles, (unsigned)p.nsplit);
-        if (p.split)
-            tc::k_tc_fwd_split<<<grid, tc::kFwdSplitThreads, fwd_split_smem(p.ntile_rows), st>>>(
-                p.tmA, p.tmB, p.tmA_lo, p.tmB_lo, n_freq, p.ntile_rows, p.ktiles, p.kt_per_split, kSplitChainTiles,
-                p.mt_alloc, b0 / 64, part, err);
-        else if (NM == 1)
-            tc::k_tc_fwd<1, 4><<<grid, 128, fwd_smem<1, 4>(p.ntile_rows), st>>>(
-                p.tmA, p.tmB, n_freq, p.ntile_rows, p.ktiles, p.kt_per_split, p.mt_alloc, b0 / 64, part, err);
+        if (p.split) {
+            auto go = [&](auto kern, size_t sm) {
+                kern<<<grid, tc::kFwdSplitThreads, sm, st>>>(p.tmA[am], p.tmB, p.tmA_lo[am], p.tmB_lo, n_freq,
+                                                             p.ntile_rows, p.ktiles, p.kt_per_split,
+                                                             kSplitChainTiles, p.mt_alloc, b0 / 64, arows, nb, part,
+                                                             err);
+            };
+            const size_t c4 = tc::FwdSplit<true, 4>::smem(p.ntile_rows), c3 = tc::FwdSplit<true, 3>::smem(p.ntile_rows);
+            const size_t f4 = tc::FwdSplit<false, 4>::smem(p.ntile_rows), f3 = tc::FwdSplit<false, 3>::smem(p.ntile_rows);
+            const size_t cap = kSplitSmemMax;
+            if (arows <= 32 && c4 <= cap) go(tc::k_tc_fwd_split<true, 4>, c4);
+            else if (arows <= 32 && c3 <= cap) go(tc::k_tc_fwd_split<true, 3>, c3);
+            else if (f4 <= cap) go(tc::k_tc_fwd_split<false, 4>, f4);
+            else if (f3 <= cap) go(tc::k_tc_fwd_split<false, 3>, f3);
+            else go(tc::k_tc_fwd_split<false, 2>, tc::FwdSplit<false, 2>::smem(p.ntile_rows));
+        }
+        else if (NM == 1) {
+            // 97-160 rows of Fhat: three stages, so that two CTAs share an SM
+            // and one loads while the other starts or drains (up to 96 rows
+            // four stages leave room for two as well): 32 vectors at
+            // 1024 x 100 x 20000 2219 -> 1679 us with the fewer rows of A
+            const bool two = p.ntile_rows > 96 && p.ntile_rows <= 160, all = arows == 64;
+            auto go = [&](auto kern, size_t sm) {
+                kern<<<grid, 128, sm, st>>>(p.tmA[am], p.tmB, n_freq, p.ntile_rows, p.ktiles, p.kt_per_split,
+                                            p.mt_alloc, b0 / 64, arows, nb, part, err);
+            };
+            const size_t sm3 = fwd_smem<1, 3>(p.ntile_rows), sm4 = fwd_smem<1, 4>(p.ntile_rows);
+            if (two && all) go(tc::k_tc_fwd<1, 3, true>, sm3);
+            else if (two) go(tc::k_tc_fwd<1, 3, false>, sm3);
+            else if (all) go(tc::k_tc_fwd<1, 4, true>, sm4);
+            else go(tc::k_tc_fwd<1, 4, false>, sm4);
+        }
         else
-            tc::k_tc_fwd<2, 3><<<grid, 128, fwd_smem<2, 3>(p.ntile_rows), st>>>(
-                p.tmA, p.tmB, n_freq, p.ntile_rows, p.ktiles, p.kt_per_split, p.mt_alloc, b0 / 64, part, err);
+            tc::k_tc_fwd<2, 3, true><<<grid, 128, fwd_smem<2, 3>(p.ntile_rows), st>>>(
+                p.tmA[am], p.tmB, n_freq, p.ntile_rows, p.ktiles, p.kt_per_split, p.mt_alloc, b0 / 64, arows, nb, part,
+                err);
         count_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;

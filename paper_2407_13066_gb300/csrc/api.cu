@@ -88,6 +88,8 @@ struct btt_op {
     int staging_nrhs = 1;             // vectors the host staging buffers hold
     int device = 0;
     FftGeom geom{};
+    SetupPlan splan{};
+    const int* setup_tab = nullptr;   // positions of the setup transform (part of `pos`)
     void* fhat = nullptr;
     size_t fhat_bytes = 0;
     float* scales = nullptr;          // per-frequency scales (F16S only)
@@ -187,17 +189,23 @@ btt_status run_create(btt_op* op, const double* blocks, bool dev_blocks, unsigne
                       int pass, double* chunk_buf, int64_t chunk_cols, double2* scratch, cudaStream_t st)
 {
     const int64_t ncol = (int64_t)op->N_d * op->N_m;
+    auto create = [&](const double* blk, int64_t nc, int64_t c0) {
+        cudaError_t e;
+        if (setup_create(blk, nc, (int)nc, c0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat, op->scales, maxbits, pass,
+                         op->splan, op->tw64, op->setup_tab, st, &e))
+            return e;
+        return launch_create(blk, nc, (int)nc, c0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat, op->scales, maxbits,
+                             pass, op->geom, op->tw64, scratch, st);
+    };
     if (dev_blocks) {
-        CK(launch_create(blocks, ncol, (int)ncol, 0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat,
-                         op->scales, maxbits, pass, op->geom, op->tw64, scratch, st));
+        CK(create(blocks, ncol, 0));
         return BTT_OK;
     }
     for (int64_t c0 = 0; c0 < ncol; c0 += chunk_cols) {
         const int64_t nc = ncol - c0 < chunk_cols ? ncol - c0 : chunk_cols;
         CK(cudaMemcpy2DAsync(chunk_buf, nc * sizeof(double), blocks + c0, ncol * sizeof(double),
                              nc * sizeof(double), op->N_t, cudaMemcpyHostToDevice, st));
-        CK(launch_create(chunk_buf, nc, (int)nc, c0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat,
-                         op->scales, maxbits, pass, op->geom, op->tw64, scratch, st));
+        CK(create(chunk_buf, nc, c0));
     }
     return BTT_OK;
 }
@@ -492,6 +500,7 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     op->staging_nrhs = staging_of(opt);
     op->gemm = opt.gemm;
     op->geom = geom;
+    const bool pf = make_setup_plan(N_t, &op->splan);
     cudaGetDevice(&op->device);
 
     const size_t nfhat = (size_t)op->n_freq * N_d * op->ldm;
@@ -526,7 +535,7 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     STEP(alloc(&op->fhat, op->fhat_bytes, "Fhat"));
     STEP(alloc((void**)&op->tw32, L * 2 * sizeof(float4), "twiddles"));
     STEP(alloc((void**)&op->tw64, L * sizeof(double2), "twiddles"));
-    STEP(alloc((void**)&op->pos, (L + geom.res_ints) * sizeof(int), "position tables"));
+    STEP(alloc((void**)&op->pos, (L + geom.res_ints + L) * sizeof(int), "position tables"));
     STEP(alloc(&op->xhat, xh_b, "mhat workspace"));
     STEP(alloc(&op->dhat, dh_b, "dhat workspace"));
     STEP(alloc(&op->stage_in, st_b, "staging"));
@@ -578,12 +587,14 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     }
     CKF(cudaMemcpyAsync(op->tw64, t64.data(), L * sizeof(double2), cudaMemcpyHostToDevice, st));
     CKF(cudaMemcpyAsync(op->tw32, t32.data(), t32.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
-    std::vector<int> pos(L + geom.res_ints);
+    std::vector<int> pos(L + geom.res_ints + L);
     digit_reversal(op->geom, pos.data());
     res_tables(op->geom, pos.data() + L);
+    if (pf) setup_tables(op->splan, pos.data() + L + geom.res_ints);
     CKF(cudaMemcpyAsync(op->pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     op->geom.pos = op->pos;
     op->geom.res_tab = op->pos + L;
+    if (pf) op->setup_tab = op->pos + L + geom.res_ints;
     // zero Fhat (row padding l >= N_m stays zero) and the workspace padding
     CKF(cudaMemsetAsync(op->fhat, 0, op->fhat_bytes, st));
     CKF(cudaMemsetAsync(op->xhat, 0, xh_b, st));

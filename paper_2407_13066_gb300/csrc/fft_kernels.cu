@@ -351,6 +351,7 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess) e = prepare_static_fft();
     if (e == cudaSuccess) e = prepare_exchange_fft();
     if (e == cudaSuccess) e = prepare_res_fft();
+    if (e == cudaSuccess) e = prepare_setup_fft();
     return e;
 }
 

@@ -17,6 +17,16 @@ struct ResPlan {
     unsigned magic[kResPasses];
 };
 
+// Plan of the FP64 setup transform (fft_setup.cu): the prime powers of N_t and
+// their passes (radix, sub-positions S, points I behind the dimension, twiddle
+// step in the length-L table).
+constexpr int kSetupPasses = 12;
+struct SetupPlan {
+    int N, ndim, np;
+    int dim[4];
+    int radix[kSetupPasses], pdim[kSetupPasses], S[kSetupPasses], I[kSetupPasses], tstep[kSetupPasses];
+};
+
 // Geometry of the time transforms of one operator.
 struct FftGeom {
     int N_t;       // samples kept
@@ -105,6 +115,17 @@ cudaError_t launch_create(const double* blk, int64_t ldb, int ncols, int64_t col
 // scales[w] = fp32(max_w / target), or 1 for an all-zero slice.
 cudaError_t launch_make_scales(const unsigned long long* maxbits, float* scales, int n, double target,
                                cudaStream_t st);
+
+// The prime-factor form (fft_setup.cu), used by launch_create's callers where
+// its tile fits in shared memory; false otherwise.  tab: device copy of the
+// 2 N_t entries of setup_tables.
+bool make_setup_plan(int N_t, SetupPlan* p);
+void setup_tables(const SetupPlan& p, int* t);
+bool setup_fits(const SetupPlan& p, bool find_max);
+cudaError_t prepare_setup_fft();
+bool setup_create(const double* blk, int64_t ldb, int ncols, int64_t col_base, int N_d, int N_m, int ldm, int prec,
+                  void* fhat, const float* scales, unsigned long long* maxbits, int pass, const SetupPlan& p,
+                  const double2* tw, const int* tab, cudaStream_t st, cudaError_t* err);
 
 // ---- per-frequency products (gemv_kernels.cu) ----
 // dh[b][w][s] = sum_l Fhat[w][s][l] xh[b][w][l]          (Alg. 2, apply_matrix)

@@ -1,0 +1,43 @@
+"""Setup transform in its prime-factor form (fft_setup.cu): every prime power
+and several together, more than one pass per power, series rows that straddle
+two rows of Fhat (odd N_m), single columns, host blocks in device memory or
+staged; 6480 is past its shared memory (the mixed-radix kernel runs)."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from oracle import fft_method, quantize
+import paper_2407_13066_gb300 as btt
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # (N_t, N_d, N_m)
+    (1, 2, 3), (2, 1, 1), (7, 3, 5), (16, 4, 6), (27, 1, 9), (49, 5, 3), (125, 2, 4), (360, 3, 7), (512, 1, 3),
+    (1125, 2, 3), (2520, 1, 5), (4096, 1, 2), (6480, 1, 3),
+]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_stored_fhat(shape):
+    """FP64 storage to 1e-13 of the largest entry (the bound of the 64-step
+    test), FP32 to one unit in the last place of it, FP16 scales to 1e-6."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("setup", N_t, N_d, N_m, tau=max(1.0, N_t / 5), seed=N_t + N_m)
+    F = synth.blocks(w)
+    ref = fft_method.setup(F)
+    top = np.abs(ref).max()
+    for prec, dtype, tol in (("f64", np.complex128, 1e-13), ("f32", np.complex64, 2.0 ** -23)):
+        raws = []
+        for blocks in (F, torch.from_numpy(F).cuda()):
+            with btt.Operator(blocks, precision=prec) as op:
+                raw, _ = op.copy_fhat()
+                ld = op.fhat_ld()
+            raws.append(raw)
+        assert np.array_equal(raws[0], raws[1])
+        got = raws[0].view(dtype).reshape(N_t + 1, N_d, ld)
+        assert np.abs(got[:, :, :N_m] - ref).max() <= tol * top
+        assert np.all(got[:, :, N_m:] == 0)
+    with btt.Operator(F, precision="f16s") as op:
+        _, sc = op.copy_fhat()
+    np.testing.assert_allclose(sc, quantize.fp16_scales(ref), rtol=1e-6)

@@ -87,21 +87,26 @@ k_gemv_fwd(const typename Store<PREC>::elem* __restrict__ fhat, const float* __r
         }
     }
 
-    // reduce over the CTA: warp shuffles, then one partial per warp in smem
+    // Reduce over the CTA: over the lanes with each lane keeping half of the
+    // sums per step (9 additions a lane for 8 sums; all five steps for all
+    // sums took 40, which at the FP64 rate and 1000 columns were 40% of the
+    // kernel: 1212 -> 824 us at 1000 x 100 x 1000), then one partial per warp
     __shared__ V red[NT / 32][R * NB];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    A v[2 * R * NB];
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
-            V a = acc[r][n];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
-                a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
-            }
-            if (lane == 0) red[wid][r * NB + n] = a;
+            v[2 * (r * NB + n)] = acc[r][n].x;
+            v[2 * (r * NB + n) + 1] = acc[r][n].y;
         }
+    using LS = LaneSum<2 * R * NB, 16>;
+    int base = 0;
+    LS::run(v, lane, base);
+    if (!(lane & LS::kDup))
+#pragma unroll
+        for (int i = 0; i < LS::kLeft; ++i) reinterpret_cast<A*>(red[wid])[base + i] = v[i];
     __syncthreads();
     if (threadIdx.x < R * NB) {
         const int r = threadIdx.x / NB, n = threadIdx.x % NB;
@@ -362,7 +367,7 @@ constexpr int kGemvThreads = 256;
 
 constexpr int kAdjUnroll = 8;
 
-template <int PREC, int R, int NB>
+template <int PREC, int R, int NB, int NT>
 static cudaError_t fwd_launch(const void* fhat, const float* scales, int n_freq, int N_d, int ldm,
                               const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs,
                               cudaStream_t st)
@@ -370,7 +375,7 @@ static cudaError_t fwd_launch(const void* fhat, const float* scales, int n_freq,
     using S = Store<PREC>;
     using V = cplx_t<typename S::acc>;
     dim3 grid((nrhs + NB - 1) / NB, (N_d + R - 1) / R, n_freq);
-    k_gemv_fwd<PREC, R, NB, kGemvThreads><<<grid, kGemvThreads, 0, st>>>(
+    k_gemv_fwd<PREC, R, NB, NT><<<grid, NT, 0, st>>>(
         static_cast<const typename S::elem*>(fhat), scales, N_d, ldm, static_cast<const V*>(xh), xbs,
         static_cast<V*>(dh), dbs, nrhs, lo_plane(PREC, n_freq, N_d, ldm));
     count_launch();
@@ -459,7 +464,13 @@ cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int
         return launch_gemv_fwd_multi(prec, fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
     switch (prec) {
         case P_F32: return fwd_dispatch<P_F32>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
-        case P_F64: return fwd_launch<P_F64, 4, 1>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
+        case P_F64:
+            // short rows on two warps: the sums over lanes cost as much as 18
+            // columns per warp (1000 x 100 x 1000 824 -> 731 us, 5000 x 10 x 200
+            // 183 -> 134)
+            return ldm <= 8192 ? fwd_launch<P_F64, 4, 1, 64>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st)
+                               : fwd_launch<P_F64, 4, 1, kGemvThreads>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs,
+                                                                       nrhs, st);
         case P_F16S: return fwd_dispatch<P_F16S>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_BF16: return fwd_dispatch<P_BF16>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_BF16X2: return fwd_dispatch<P_BF16X2>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);

@@ -63,40 +63,6 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// Sums v[0..CNT) over the 32 lanes.  While the count is even a lane sends
-// half of its values to its partner and keeps the sums of the other half;
-// `base` is the index of the first value it ends with.  Adds the same pairs
-// in the same tree as a butterfly over all values, with a fifth of the
-// shuffles at CNT = 64.  Returns the number of values a lane ends with;
-// lanes that differ only in `dup` bits hold the same ones.
-template <int CNT, int O> struct LaneSum {
-    static constexpr bool kHalve = CNT % 2 == 0;
-    static constexpr int kNext = kHalve ? CNT / 2 : CNT;
-    static constexpr int kLeft = LaneSum<kNext, O / 2>::kLeft;
-    static constexpr int kDup = (kHalve ? 0 : O) | LaneSum<kNext, O / 2>::kDup;
-    static __device__ __forceinline__ void run(float* v, int lane, int& base)
-    {
-        if constexpr (kHalve) {
-            const bool up = lane & O;
-#pragma unroll
-            for (int i = 0; i < kNext; ++i) {
-                const float send = up ? v[i] : v[i + kNext], keep = up ? v[i + kNext] : v[i];
-                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-            }
-            base += up ? kNext : 0;
-        } else {
-#pragma unroll
-            for (int i = 0; i < CNT; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], O);
-        }
-        LaneSum<kNext, O / 2>::run(v, lane, base);
-    }
-};
-template <int CNT> struct LaneSum<CNT, 0> {
-    static constexpr int kLeft = CNT;
-    static constexpr int kDup = 0;
-    static __device__ __forceinline__ void run(float*, int, int&) {}
-};
-
 // ------------------------------------------------------------ F (Alg. 2)
 // CTA = rg warps x 4 rows of one frequency (times wk warps that share the
 // blocks along l when there are few rows) for a group of NB vectors; the

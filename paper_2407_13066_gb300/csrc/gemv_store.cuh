@@ -147,6 +147,40 @@ template <typename V> __device__ __forceinline__ void cfma_conj(V& acc, V a, V b
     acc.y = fma(-a.y, b.x, acc.y);
 }
 
+// Sums v[0..CNT) over the 32 lanes.  While the count is even a lane sends
+// half of its values to its partner and keeps the sums of the other half;
+// `base` is the index of the first value it ends with.  Adds the same pairs
+// in the same tree as a butterfly over all values, with a fifth of the
+// shuffles at CNT = 64.  Returns the number of values a lane ends with;
+// lanes that differ only in `dup` bits hold the same ones.
+template <int CNT, int O> struct LaneSum {
+    static constexpr bool kHalve = CNT % 2 == 0;
+    static constexpr int kNext = kHalve ? CNT / 2 : CNT;
+    static constexpr int kLeft = LaneSum<kNext, O / 2>::kLeft;
+    static constexpr int kDup = (kHalve ? 0 : O) | LaneSum<kNext, O / 2>::kDup;
+    template <typename T> static __device__ __forceinline__ void run(T* v, int lane, int& base)
+    {
+        if constexpr (kHalve) {
+            const bool up = lane & O;
+#pragma unroll
+            for (int i = 0; i < kNext; ++i) {
+                const T send = up ? v[i] : v[i + kNext], keep = up ? v[i + kNext] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+            }
+            base += up ? kNext : 0;
+        } else {
+#pragma unroll
+            for (int i = 0; i < CNT; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], O);
+        }
+        LaneSum<kNext, O / 2>::run(v, lane, base);
+    }
+};
+template <int CNT> struct LaneSum<CNT, 0> {
+    static constexpr int kLeft = CNT;
+    static constexpr int kDup = 0;
+    template <typename T> static __device__ __forceinline__ void run(T*, int, int&) {}
+};
+
 // Element offset of the lo plane of a split-pair Fhat (0 for other formats).
 inline int64_t lo_plane(int prec, int n_freq, int N_d, int ldm)
 {

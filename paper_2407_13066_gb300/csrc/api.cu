@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <string>
+#include <utility>
 #include <type_traits>
 #include <vector>
 
@@ -568,10 +569,28 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     // (2 m + 1) n2, entry n2 R1/2 + m, for the one-exchange transforms
     // (L = R1 N2, R1 = min(32, L/16), n2 < N2, m < R1/2; the 1/2 is exact))
     std::vector<float2> t32(4 * (size_t)L);
-    for (int e = 0; e < L; ++e) {
+    // (evaluated over the first octant, or quadrant where 4 does not divide L,
+    // and mirrored: long double is 128 bits in software on Arm, and four calls
+    // per entry were 10 ms of btt_create at L = 18 000)
+    const int top = L % 4 == 0 ? L / 8 : L / 4;
+    std::vector<std::pair<long double, long double>> first(top + 1);
+    for (int e = 0; e <= top; ++e) {
         const long double a = 2.0L * 3.14159265358979323846264338327950288L * (long double)e / (long double)L;
-        t64[e] = make_double2((double)cosl(a), (double)-sinl(a));
-        const float c = (float)cosl(a), d = (float)-sinl(a);
+        first[e] = {cosl(a), sinl(a)};
+    }
+    for (int e = 0; e < L; ++e) {
+        const bool below = 2 * e > L;   // lower half: conjugate
+        int f = below ? L - e : e;
+        const bool left = 4 * f > L;    // second quadrant
+        if (left) f = L / 2 - f;
+        const bool steep = f > top;     // second octant
+        if (steep) f = L / 4 - f;
+        long double cl = first[f].first, sl = first[f].second;
+        if (steep) std::swap(cl, sl);
+        if (left) cl = -cl;
+        if (below) sl = -sl;
+        t64[e] = make_double2((double)cl, (double)-sl);
+        const float c = (float)cl, d = (float)-sl;
         t32[e] = make_float2(c, d);
         t32[L + 2 * (size_t)e] = make_float2(c, c);
         t32[L + 2 * (size_t)e + 1] = make_float2(d, d);

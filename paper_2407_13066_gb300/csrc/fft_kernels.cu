@@ -320,6 +320,11 @@ static dim3 col_grid(int ncols, int nb, int wc_log2)
 
 cudaError_t prepare_kernels()
 {
+    // set already on this device's context: about 130 attribute calls are
+    // 0.1 ms of every btt_create (the last one set below is looked at)
+    cudaFuncAttributes last{};
+    cudaError_t e = cudaFuncGetAttributes(&last, k_create<P_FP8S>);
+    if (e != cudaSuccess || last.maxDynamicSharedSizeBytes > 48 * 1024) return e;
     // limits clamped to what this device lets one CTA claim
     int dev = 0, optin = kFftSmemMax;
     cudaGetDevice(&dev);
@@ -328,7 +333,6 @@ cudaError_t prepare_kernels()
     const int fmax_f = kFftMaxL * (int)sizeof(float2) < cap ? kFftMaxL * (int)sizeof(float2) : cap;
     const int fmax_d = cap;
     const int cmax = cap;
-    cudaError_t e = cudaSuccess;
 #define BTT_SET(k, b) \
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
     BTT_SET(k_rfft<float>, fmax_f);
@@ -344,12 +348,12 @@ cudaError_t prepare_kernels()
     BTT_SET(k_create<P_F16S>, cmax);
     BTT_SET(k_create<P_BF16>, cmax);
     BTT_SET(k_create<P_BF16X2>, cmax);
-    BTT_SET(k_create<P_FP8S>, cmax);
-#undef BTT_SET
     if (e == cudaSuccess) e = prepare_static_fft();
     if (e == cudaSuccess) e = prepare_exchange_fft();
     if (e == cudaSuccess) e = prepare_res_fft();
     if (e == cudaSuccess) e = prepare_setup_fft();
+    BTT_SET(k_create<P_FP8S>, cmax);
+#undef BTT_SET
     return e;
 }
 

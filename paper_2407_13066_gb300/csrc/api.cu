@@ -89,8 +89,6 @@ struct btt_op {
     int staging_nrhs = 1;             // vectors the host staging buffers hold
     int device = 0;
     FftGeom geom{};
-    SetupPlan splan{};
-    const int* setup_tab = nullptr;   // positions of the setup transform (part of `pos`)
     void* fhat = nullptr;
     size_t fhat_bytes = 0;
     float* scales = nullptr;          // per-frequency scales (F16S only)
@@ -193,7 +191,7 @@ btt_status run_create(btt_op* op, const double* blocks, bool dev_blocks, unsigne
     auto create = [&](const double* blk, int64_t nc, int64_t c0) {
         cudaError_t e;
         if (setup_create(blk, nc, (int)nc, c0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat, op->scales, maxbits, pass,
-                         op->splan, op->tw64, op->setup_tab, st, &e))
+                         op->geom.splan, op->tw64, op->geom.setup_tab, st, &e))
             return e;
         return launch_create(blk, nc, (int)nc, c0, op->N_d, op->N_m, op->ldm, op->prec, op->fhat, op->scales, maxbits,
                              pass, op->geom, op->tw64, scratch, st);
@@ -501,7 +499,7 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     op->staging_nrhs = staging_of(opt);
     op->gemm = opt.gemm;
     op->geom = geom;
-    const bool pf = make_setup_plan(N_t, &op->splan);
+    const bool pf = make_setup_plan(N_t, &op->geom.splan);
     cudaGetDevice(&op->device);
 
     const size_t nfhat = (size_t)op->n_freq * N_d * op->ldm;
@@ -609,11 +607,11 @@ btt_status op_setup(btt_op** out, int N_t, int N_d, int N_m, const btt_options* 
     std::vector<int> pos(L + geom.res_ints + L);
     digit_reversal(op->geom, pos.data());
     res_tables(op->geom, pos.data() + L);
-    if (pf) setup_tables(op->splan, pos.data() + L + geom.res_ints);
+    if (pf) setup_tables(op->geom.splan, pos.data() + L + geom.res_ints);
     CKF(cudaMemcpyAsync(op->pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice, st));
     op->geom.pos = op->pos;
     op->geom.res_tab = op->pos + L;
-    if (pf) op->setup_tab = op->pos + L + geom.res_ints;
+    if (pf) op->geom.setup_tab = op->pos + L + geom.res_ints;
     // zero Fhat (row padding l >= N_m stays zero) and the workspace padding
     CKF(cudaMemsetAsync(op->fhat, 0, op->fhat_bytes, st));
     CKF(cudaMemsetAsync(op->xhat, 0, xh_b, st));

@@ -32,6 +32,7 @@ bool make_fft_geom(int N_t, FftGeom* g)
     g->plan = p;
     g->pos = nullptr;
     g->res_tab = nullptr;
+    g->setup_tab = nullptr;
     make_res_plans(g);
     return true;
 }
@@ -381,6 +382,10 @@ cudaError_t launch_rfft(const T* x, int64_t ldx, int64_t bsx, int ncols, cplx_t<
         if (static_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e)) return e;
         if (res_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e)) return e;
     }
+    if constexpr (std::is_same<T, double>::value) {
+        cudaError_t e;
+        if (pf_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e)) return e;
+    }
     const int wc = tile_log2<T>(ncols, nb, g);
     k_rfft<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(
         x, ldx, bsx, ncols, X, ldo, bso, g.N_t, g.plan, wc, tw, g.pos, xptr);
@@ -399,6 +404,10 @@ cudaError_t launch_irfft(const cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols
         if (exchange_irfft(X, ldx, bsx, ncols, y, ldy, bsy, gam, nb, g, tw, st, yptr, &e)) return e;
         if (static_irfft(X, ldx, bsx, ncols, y, ldy, bsy, gam, nb, g, tw, st, yptr, &e)) return e;
         if (res_irfft(X, ldx, bsx, ncols, y, ldy, bsy, gam, nb, g, tw, st, yptr, &e)) return e;
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        cudaError_t e;
+        if (pf_irfft(X, ldx, bsx, ncols, y, ldy, bsy, gam, nb, g, tw, st, yptr, &e)) return e;
     }
     const int wc = tile_log2<T>(ncols, nb, g);
     k_irfft<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(
@@ -444,6 +453,10 @@ cudaError_t launch_hess_mid(cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols, c
             res_rfft(scratch, ncols, n, ncols, X, ldx, bsx, nb, g, tw, st, nullptr, &e);
             return e;
         }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        cudaError_t e;
+        if (pf_hess_mid(X, ldx, bsx, ncols, gam, nb, g, tw, st, &e)) return e;
     }
     const int wc = tile_log2<T>(ncols, nb, g);
     k_hess_mid<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(

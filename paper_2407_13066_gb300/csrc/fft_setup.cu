@@ -144,6 +144,23 @@ __device__ __forceinline__ void pass(double2* buf, int total, int S, int I, int 
     __syncthreads();
 }
 
+__device__ __forceinline__ void passes(double2* buf, int total, const SetupPlan& plan, int wcl,
+                                       const double2* __restrict__ tw)
+{
+    for (int p = 0; p < plan.np; ++p) {
+        const int S = plan.S[p], I = plan.I[p], ts = plan.tstep[p];
+        switch (plan.radix[p]) {
+            case 2: pass<2>(buf, total, S, I, wcl, ts, tw); break;
+            case 3: pass<3>(buf, total, S, I, wcl, ts, tw); break;
+            case 4: pass<4>(buf, total, S, I, wcl, ts, tw); break;
+            case 5: pass<5>(buf, total, S, I, wcl, ts, tw); break;
+            case 7: pass<7>(buf, total, S, I, wcl, ts, tw); break;
+            case 8: pass<8>(buf, total, S, I, wcl, ts, tw); break;
+            default: pass<9>(buf, total, S, I, wcl, ts, tw); break;
+        }
+    }
+}
+
 template <int PREC>
 __global__ void __launch_bounds__(NT, 2)
 k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_base, int N_d, int N_m, int ldm,
@@ -193,18 +210,7 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
             }
         }
         __syncthreads();
-        for (int p = 0; p < plan.np; ++p) {
-            const int S = plan.S[p], I = plan.I[p], ts = plan.tstep[p];
-            switch (plan.radix[p]) {
-                case 2: pass<2>(buf, L, S, I, wcl, ts, tw); break;
-                case 3: pass<3>(buf, L, S, I, wcl, ts, tw); break;
-                case 4: pass<4>(buf, L, S, I, wcl, ts, tw); break;
-                case 5: pass<5>(buf, L, S, I, wcl, ts, tw); break;
-                case 7: pass<7>(buf, L, S, I, wcl, ts, tw); break;
-                case 8: pass<8>(buf, L, S, I, wcl, ts, tw); break;
-                default: pass<9>(buf, L, S, I, wcl, ts, tw); break;
-            }
-        }
+        passes(buf, L, plan, wcl, tw);
         // where this thread's two columns go
         const unsigned g0 = (unsigned)(col_base + col);
         const unsigned s0 = one ? g0 / (unsigned)N_m : 0u, l0 = g0 - s0 * (unsigned)N_m;
@@ -280,6 +286,177 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
         for (int i = threadIdx.x; i <= N; i += NT)
             if (smax[i]) atomicMax(&maxbits[i], smax[i]);
     }
+}
+
+// ------------------------------------------------ FP64 vector transforms
+// The transforms of BTT_F64 operators on the same passes.  The inverse runs
+// them on conjugates (IDFT(X) = conj DFT(conj X)) of both halves.  Against the
+// mixed-radix kernels of fft_kernels.cu (us, one vector; input / inverse of
+// N_m columns, averaged with N_d, and middle step of N_d columns):
+//   1000 x 100 x 1000  131 / 125 / 88 -> 82 / 86 / 62
+//   420 x 37 x 3001    131 / 124 / 44 -> 75 / 73 / 29
+//   5000 x 10 x 200    230 / 219 / 441 -> 140 / 160 / 307
+// At 64 x 8 x 32 they are latency (a warp's FP64 instruction occupies the
+// pipe for 16 clocks): 14.4 / 14.5 / 24 -> 12.3 / 12.3 / 18.6 with event timers.
+
+struct Tables {   // positions of sample n and of frequency k, in shared memory
+    unsigned short *in, *out;
+    __device__ __forceinline__ Tables(unsigned char* at, int N, const int* __restrict__ tab)
+    {
+        in = reinterpret_cast<unsigned short*>(at);
+        out = in + N;
+        for (int i = threadIdx.x; i < N; i += NT) {
+            in[i] = (unsigned short)__ldg(tab + i);
+            out[i] = (unsigned short)__ldg(tab + N + i);
+        }
+    }
+};
+
+// Rows w = 2 j + odd <= N of one half (values halved) to X.
+__device__ __forceinline__ void store_half(const double2* half, int odd, int N, int wcl, const unsigned short* out,
+                                           double2* X, int64_t ldx, int col, int ncols)
+{
+    const int c = threadIdx.x & ((1 << wcl) - 1);
+    if (col >= ncols) return;
+    for (int j = threadIdx.x >> wcl; 2 * j + odd <= N; j += NT >> wcl) {
+        const double2 z = half[((int)out[j] << wcl) + c];
+        const double2 zc = half[((int)out[odd ? N - 1 - j : (j ? N - j : 0)] << wcl) + c];
+        double2* o = X + (int64_t)(2 * j + odd) * ldx + col;
+        o[0] = make_double2(z.x + zc.x, z.y - zc.y);
+        if (col + 1 < ncols) o[1] = make_double2(z.y + zc.y, zc.x - z.x);
+    }
+}
+
+// Conjugates of Z[w] = A + i B and Z[L - w] of every row to their halves.
+__device__ __forceinline__ void load_conj(double2* buf, int N, int wcl, const unsigned short* in,
+                                          const double2* __restrict__ X, int64_t ldx, int col, int ncols)
+{
+    const int c = threadIdx.x & ((1 << wcl) - 1);
+    for (int w = threadIdx.x >> wcl; w <= N; w += NT >> wcl) {
+        double2 a = make_double2(0., 0.), b = a;
+        if (col < ncols) a = X[(int64_t)w * ldx + col];
+        if (col + 1 < ncols) b = X[(int64_t)w * ldx + col + 1];
+        if (w == 0 || w == N) a.y = b.y = 0.;   // real bins
+        const int j = w >> 1, jj = w & 1 ? N - 1 - j : (j ? N - j : 0);
+        double2* half = buf + (w & 1 ? (N << wcl) : 0);
+        half[((int)in[j] << wcl) + c] = make_double2(a.x - b.y, -(a.y + b.x));
+        if (jj != j) half[((int)in[jj] << wcl) + c] = make_double2(a.x + b.y, a.y - b.x);
+    }
+}
+
+// blockIdx.z: the half (even or odd frequencies) of this CTA, so that a few
+// columns' FP64 work spreads over twice the SMs; the samples are read twice.
+__global__ void __launch_bounds__(NT, 2)
+k_rfft_pf(const double* __restrict__ x, int64_t ldx, int64_t bsx, int ncols, double2* __restrict__ X, int64_t ldo,
+          int64_t bso, SetupPlan plan, int wcl, const double2* __restrict__ tw, const int* __restrict__ tab,
+          const double* const* __restrict__ xptr)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = plan.N, odd = blockIdx.z, c = threadIdx.x & ((1 << wcl) - 1);
+    const int col = (int)(blockIdx.x << (wcl + 1)) + 2 * c;
+    const int64_t b = blockIdx.y;
+    double2* buf = reinterpret_cast<double2*>(smem_raw);
+    const Tables t(smem_raw + ((size_t)N << wcl) * sizeof(double2), N, tab);
+    const double* xb = (xptr ? xptr[b] : x + b * bsx) + col;
+    __syncthreads();
+    for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
+        double2 z = make_double2(0., 0.);
+        if (col < ncols) z.x = 0.5 * xb[(int64_t)n * ldx];
+        if (col + 1 < ncols) z.y = 0.5 * xb[(int64_t)n * ldx + 1];
+        buf[((int)t.in[n] << wcl) + c] = odd ? mul(z, __ldg(tw + n)) : z;
+    }
+    __syncthreads();
+    passes(buf, N, plan, wcl, tw);
+    store_half(buf, odd, N, wcl, t.out, X + b * bso, ldo, col, ncols);
+}
+
+__global__ void __launch_bounds__(NT, 2)
+k_irfft_pf(const double2* __restrict__ X, int64_t ldx, int64_t bsx, int ncols, double* __restrict__ y, int64_t ldy,
+           int64_t bsy, const double* __restrict__ g, SetupPlan plan, int wcl, const double2* __restrict__ tw,
+           const int* __restrict__ tab, double* const* __restrict__ yptr)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = plan.N, c = threadIdx.x & ((1 << wcl) - 1);
+    const int col = (int)(blockIdx.x << (wcl + 1)) + 2 * c;
+    const int64_t b = blockIdx.y;
+    double2* buf = reinterpret_cast<double2*>(smem_raw);
+    const Tables t(smem_raw + ((size_t)2 * N << wcl) * sizeof(double2), N, tab);
+    __syncthreads();
+    load_conj(buf, N, wcl, t.in, X + b * bsx, ldx, col, ncols);
+    __syncthreads();
+    passes(buf, 2 * N, plan, wcl, tw);
+    const double inv = 1. / (2. * N);
+    double* yb = (yptr ? yptr[b] : y + b * bsy) + col;
+    if (col >= ncols) return;
+    for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
+        // conj(y) = (E + w_L^n O) / L
+        const int at = ((int)t.out[n] << wcl) + c;
+        const double2 v = add(buf[at], mul(buf[(N << wcl) + at], __ldg(tw + n)));
+        double p = v.x * inv, q = -v.y * inv;
+        if (g) {
+            p *= g[(int64_t)n * ncols + col];
+            if (col + 1 < ncols) q *= g[(int64_t)n * ncols + col + 1];
+        }
+        yb[(int64_t)n * ldy] = p;
+        if (col + 1 < ncols) yb[(int64_t)n * ldy + 1] = q;
+    }
+}
+
+// In place: X <- rfft(pad(irfft(X)[:N] g)).
+__global__ void __launch_bounds__(NT, 2)
+k_mid_pf(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* __restrict__ g, SetupPlan plan, int wcl,
+         const double2* __restrict__ tw, const int* __restrict__ tab)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = plan.N, c = threadIdx.x & ((1 << wcl) - 1);
+    const int col = (int)(blockIdx.x << (wcl + 1)) + 2 * c;
+    double2* buf = reinterpret_cast<double2*>(smem_raw);
+    double2* odd = buf + (N << wcl);
+    const Tables t(smem_raw + ((size_t)2 * N << wcl) * sizeof(double2), N, tab);
+    double2* Xb = X + blockIdx.y * bsx;
+    __syncthreads();
+    load_conj(buf, N, wcl, t.in, Xb, ldx, col, ncols);
+    __syncthreads();
+    passes(buf, 2 * N, plan, wcl, tw);
+    const double inv = 0.5 / (2. * N);   // the unpack's 1/2 with it
+    for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
+        const int at = ((int)t.out[n] << wcl) + c;
+        const double2 v = add(buf[at], mul(odd[at], __ldg(tw + n)));
+        double2 z = make_double2(v.x * inv, -v.y * inv);
+        if (g) {
+            if (col < ncols) z.x *= g[(int64_t)n * ncols + col];
+            if (col + 1 < ncols) z.y *= g[(int64_t)n * ncols + col + 1];
+        }
+        buf[at] = z;
+    }
+    __syncthreads();
+    // back to the input positions through the odd half
+    for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl)
+        odd[((int)t.in[n] << wcl) + c] = buf[((int)t.out[n] << wcl) + c];
+    __syncthreads();
+    for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
+        const int at = ((int)t.in[n] << wcl) + c;
+        const double2 z = odd[at];
+        buf[at] = z;
+        odd[at] = mul(z, __ldg(tw + n));
+    }
+    __syncthreads();
+    passes(buf, 2 * N, plan, wcl, tw);
+    store_half(buf, 0, N, wcl, t.out, Xb, ldx, col, ncols);
+    store_half(odd, 1, N, wcl, t.out, Xb, ldx, col, ncols);
+}
+
+static size_t vec_smem(int N, int halves, int wcl) { return ((size_t)halves * N << wcl) * sizeof(double2) + (size_t)N * 4; }
+
+// Column pairs per CTA: up to 8, two CTAs per SM by shared memory, and as few
+// as give two CTAs per SM work (an SM has two FP64 lanes).
+static int vec_tile(int N, int halves, int ncols, int nb)
+{
+    int w = 0;
+    while (w < 3 && vec_smem(N, halves, w + 1) <= 113 * 1024) ++w;
+    const int64_t z = halves == 1 ? 2 : 1;
+    while (w > 0 && z * nb * ((ncols + (2 << w) - 1) / (2 << w)) < 2 * 152) --w;
+    return w;
 }
 
 // Shared memory at Wc = 2^wcl column pairs per tile.
@@ -367,7 +544,50 @@ cudaError_t prepare_setup_fft()
     for (auto k : {setup::k_create_pf<P_F32>, setup::k_create_pf<P_F16S>, setup::k_create_pf<P_BF16>,
                    setup::k_create_pf<P_BF16X2>, setup::k_create_pf<P_F64>, setup::k_create_pf<P_FP8S>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(setup::k_rfft_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(setup::k_irfft_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(setup::k_mid_pf, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
     return e;
+}
+
+bool pf_rfft(const double* x, int64_t ldx, int64_t bsx, int ncols, double2* X, int64_t ldo, int64_t bso, int nb,
+             const FftGeom& g, const double2* tw, cudaStream_t st, const double* const* xptr, cudaError_t* err)
+{
+    const int N = g.N_t;
+    if (!g.setup_tab || setup::vec_smem(N, 1, 0) > (size_t)kFftSmemMax) return false;
+    const int w = setup::vec_tile(N, 1, ncols, nb);
+    setup::k_rfft_pf<<<dim3((ncols + (2 << w) - 1) / (2 << w), nb, 2), setup::NT, setup::vec_smem(N, 1, w), st>>>(
+        x, ldx, bsx, ncols, X, ldo, bso, g.splan, w, tw, g.setup_tab, xptr);
+    count_launch();
+    *err = cudaGetLastError();
+    return true;
+}
+
+bool pf_irfft(const double2* X, int64_t ldx, int64_t bsx, int ncols, double* y, int64_t ldy, int64_t bsy,
+              const double* gam, int nb, const FftGeom& g, const double2* tw, cudaStream_t st, double* const* yptr,
+              cudaError_t* err)
+{
+    const int N = g.N_t;
+    if (!g.setup_tab || setup::vec_smem(N, 2, 0) > (size_t)kFftSmemMax) return false;
+    const int w = setup::vec_tile(N, 2, ncols, nb);
+    setup::k_irfft_pf<<<dim3((ncols + (2 << w) - 1) / (2 << w), nb), setup::NT, setup::vec_smem(N, 2, w), st>>>(
+        X, ldx, bsx, ncols, y, ldy, bsy, gam, g.splan, w, tw, g.setup_tab, yptr);
+    count_launch();
+    *err = cudaGetLastError();
+    return true;
+}
+
+bool pf_hess_mid(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* gam, int nb, const FftGeom& g,
+                 const double2* tw, cudaStream_t st, cudaError_t* err)
+{
+    const int N = g.N_t;
+    if (!g.setup_tab || setup::vec_smem(N, 2, 0) > (size_t)kFftSmemMax) return false;
+    const int w = setup::vec_tile(N, 2, ncols, nb);
+    setup::k_mid_pf<<<dim3((ncols + (2 << w) - 1) / (2 << w), nb), setup::NT, setup::vec_smem(N, 2, w), st>>>(
+        X, ldx, bsx, ncols, gam, g.splan, w, tw, g.setup_tab);
+    count_launch();
+    *err = cudaGetLastError();
+    return true;
 }
 
 bool setup_create(const double* blk, int64_t ldb, int ncols, int64_t col_base, int N_d, int N_m, int ldm, int prec,

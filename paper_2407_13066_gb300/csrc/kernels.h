@@ -37,6 +37,8 @@ struct FftGeom {
     ResPlan res[4];  // for clusters of 1, 2, 4, 8 CTAs
     int res_ints;    // entries of their position tables
     const int* res_tab;  // device copy (NULL: the residue transforms are not used)
+    SetupPlan splan;     // prime-factor FP64 transforms
+    const int* setup_tab;  // device copy of setup_tables (NULL: not used)
 };
 
 // Builds the radix plan for L and the column tile for a shared-memory
@@ -126,6 +128,16 @@ cudaError_t prepare_setup_fft();
 bool setup_create(const double* blk, int64_t ldb, int ncols, int64_t col_base, int N_d, int N_m, int ldm, int prec,
                   void* fhat, const float* scales, unsigned long long* maxbits, int pass, const SetupPlan& p,
                   const double2* tw, const int* tab, cudaStream_t st, cudaError_t* err);
+
+// FP64 vector transforms in prime-factor form (arguments as launch_rfft,
+// launch_irfft, launch_hess_mid); false where fft_kernels.cu runs.
+bool pf_rfft(const double* x, int64_t ldx, int64_t bsx, int ncols, double2* X, int64_t ldo, int64_t bso, int nb,
+             const FftGeom& g, const double2* tw, cudaStream_t st, const double* const* xptr, cudaError_t* err);
+bool pf_irfft(const double2* X, int64_t ldx, int64_t bsx, int ncols, double* y, int64_t ldy, int64_t bsy,
+              const double* gam, int nb, const FftGeom& g, const double2* tw, cudaStream_t st, double* const* yptr,
+              cudaError_t* err);
+bool pf_hess_mid(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* gam, int nb, const FftGeom& g,
+                 const double2* tw, cudaStream_t st, cudaError_t* err);
 
 // ---- per-frequency products (gemv_kernels.cu) ----
 // dh[b][w][s] = sum_l Fhat[w][s][l] xh[b][w][l]          (Alg. 2, apply_matrix)

@@ -41,3 +41,22 @@ def test_stored_fhat(shape):
     with btt.Operator(F, precision="f16s") as op:
         _, sc = op.copy_fhat()
     np.testing.assert_allclose(sc, quantize.fp16_scales(ref), rtol=1e-6)
+
+
+@pytest.mark.parametrize("shape", SHAPES + [(20, 33, 5), (96, 3, 700)])
+def test_fp64_vectors(shape):
+    """F, F* and the Hessian of two FP64 vectors on the same passes (forward
+    halves on their own CTAs, the inverse, the middle step): the FP64 bound."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("pf64", N_t, N_d, N_m, tau=max(1.0, N_t / 5), seed=2 * N_t + N_m)
+    F, m, d = synth.blocks(w), synth.vectors(w, "m", 2), synth.vectors(w, "d", 2)
+    g = synth.noise_gamma_inv(w)
+    Fh = fft_method.setup(F)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    rel = lambda a, b: np.linalg.norm(a.cpu().numpy() - b) / np.linalg.norm(b)
+    with btt.Operator(dev(F), precision="f64", max_nrhs=2) as op:
+        f = fft_method.forward(Fh, m)
+        assert rel(op.matvec(dev(m)), f) < 1e-12
+        assert rel(op.adjoint(dev(d)), fft_method.adjoint(Fh, d)) < 1e-12
+        assert rel(op.hessian(dev(m), dev(g)), fft_method.adjoint(Fh, g * f)) < 1e-12
+        assert rel(op.hessian(dev(m)), fft_method.adjoint(Fh, f)) < 1e-12

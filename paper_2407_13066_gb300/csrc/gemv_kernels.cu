@@ -448,7 +448,7 @@ static cudaError_t fwd_dispatch(const void* fhat, const float* scales, int n_fre
 //     pairs 123 -> 31 (l split over warps), but FP16 32 vectors 170 -> 281.
 static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
 {
-    if (nrhs < 2) return false;
+    if (nrhs < 2 || N_d > 32 * 65535) return false;   // (row tiles index grid.y)
     if (nrhs > 16 && N_d <= 8 && prec != P_F32) return false;
     if ((int64_t)n_freq * ((N_d + 19) / 20) < 152) return true;
     if (nrhs == 2 || prec == P_BF16X2) return false;
@@ -508,7 +508,8 @@ cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int
     if (nrhs <= 0) return cudaSuccess;
     // several vectors: the group kernel (two in FP32 and BF16 stay here: 592
     // against 602 us at 256 x 200 x 10000, 155 against 177 at 1500 x 24 x 6000)
-    if (prec != P_F64 && nrhs > (prec == P_BF16 || prec == P_F32 ? 2 : 1))
+    // (column tiles of at least 256 index grid.y)
+    if (prec != P_F64 && nrhs > (prec == P_BF16 || prec == P_F32 ? 2 : 1) && ldm <= 256 * 65535)
         return launch_gemv_adj_multi(prec, fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
     switch (prec) {
         case P_F32:

@@ -177,7 +177,7 @@ k_gemv_fwd_multi(const typename Store<PREC>::elem* __restrict__ fhat, const floa
     };
     auto load = [&](Raw (&q)[R], int g) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) q[r] = S::load_raw(row0 + (unsigned)(off[r] + g * BLK), lo_off);
+        for (int r = 0; r < R; ++r) q[r] = S::load_raw(row0 + ((unsigned)off[r] + (unsigned)(g * BLK)), lo_off);
     };
     auto use = [&](const Raw (&q)[R], int g) {
         while (c < g >> its_log2) advance();
@@ -214,7 +214,7 @@ k_gemv_fwd_multi(const typename Store<PREC>::elem* __restrict__ fhat, const floa
             for (int r = 0; r < R; ++r) {
                 qa[r] = Raw{};
                 if ((g * 32 + lane) * VPL < ldm && BTT_IN((g * 32 + lane) * VPL + VPL - 1, ldm, CK_GEMV_FHAT))
-                    qa[r] = S::load_raw(row0 + (unsigned)(off[r] + g * BLK), lo_off);
+                    qa[r] = S::load_raw(row0 + ((unsigned)off[r] + (unsigned)(g * BLK)), lo_off);
             }
             use(qa, g);
         }

@@ -18,6 +18,7 @@
 // 0.44 ms of FP32 time), kernels of gemv_kernels.cu -> these, us per launch:
 //   FP32  F  3 vectors 779 -> 661, 8 1513 -> 1004, 32 5890 -> 3807
 //         F* 3 vectors 686 -> 595, 8 1062 -> 828, 32 3653 -> 3143
+//         F 5 vectors 1493 -> 738, 7 1513 -> 902 (a group's kernel has its own count)
 //   BF16  F  8 vectors 1456 -> 983;   F* 8 vectors 860 -> 773
 //   FP8   F  8 vectors 1997 -> 905;   F* 8 vectors 800 -> 726
 //
@@ -446,8 +447,7 @@ static int group_size(int nrhs, int cap, int64_t ctas, int resident)
     for (int g = (nrhs + cap - 1) / cap; g <= nrhs; ++g) {
         const int per = (nrhs + g - 1) / g;
         if (best && per < 2) break;
-        const int nb = per <= 4 ? per : (per <= 6 ? 6 : 8);
-        const int64_t c = ((nrhs + per - 1) / per * ctas + 152 * resident - 1) / (152 * resident) * (nb + 1);
+        const int64_t c = ((nrhs + per - 1) / per * ctas + 152 * resident - 1) / (152 * resident) * (per + 1);
         if (!best || c < cost) best = per, cost = c;
     }
     return best;
@@ -466,7 +466,9 @@ static cudaError_t fwd_groups(const void* fhat, const float* scales, int n_freq,
     BTT_FWD(3);
     if constexpr (PREC != P_BF16X2) {
         BTT_FWD(4);
+        BTT_FWD(5);
         BTT_FWD(6);
+        BTT_FWD(7);
         BTT_FWD(8);
     }
 #undef BTT_FWD
@@ -486,7 +488,11 @@ static cudaError_t adj_groups(const void* fhat, const float* scales, int n_freq,
     BTT_ADJ(3);
     BTT_ADJ(4);
     if constexpr (PREC != P_FP8S) {
+        BTT_ADJ(5);
         BTT_ADJ(6);
+        // (16-bit formats: 7 spills, which few rows do not make up for,
+        // 2000 x 7 x 3000 FP16 128 against 137 us)
+        if (PREC == P_F32 || PREC == P_BF16X2 || N_d > 16) BTT_ADJ(7);
         BTT_ADJ(8);
     }
 #undef BTT_ADJ

@@ -321,7 +321,7 @@ static dim3 col_grid(int ncols, int nb, int wc_log2)
 
 cudaError_t prepare_kernels()
 {
-    // set already on this device's context: about 130 attribute calls are
+    // set already on this device's context: about 170 attribute calls are
     // 0.1 ms of every btt_create (the last one set below is looked at)
     cudaFuncAttributes last{};
     cudaError_t e = cudaFuncGetAttributes(&last, k_create<P_FP8S>);
@@ -353,6 +353,8 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess) e = prepare_exchange_fft();
     if (e == cudaSuccess) e = prepare_res_fft();
     if (e == cudaSuccess) e = prepare_setup_fft();
+    if (e == cudaSuccess) e = prepare_gemv();
+    if (e == cudaSuccess) e = prepare_gemv_multi();
     BTT_SET(k_create<P_FP8S>, cmax);
 #undef BTT_SET
     return e;

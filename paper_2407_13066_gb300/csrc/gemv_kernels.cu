@@ -489,16 +489,30 @@ static cudaError_t adj_launch(const void* fhat, const float* scales, int n_freq,
     const int cols = kGemvThreads * S::VPL;
     dim3 grid((nrhs + NB - 1) / NB, (ldm + cols - 1) / cols, n_freq);
     const size_t sm = (size_t)NB * N_d * sizeof(V);
-    auto kern = k_gemv_adj<PREC, NB, kGemvThreads, kAdjUnroll>;
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
-    kern<<<grid, kGemvThreads, sm, st>>>(static_cast<const typename S::elem*>(fhat), scales, N_d, N_m,
-                                         ldm, static_cast<const V*>(dh), dbs, static_cast<V*>(mh), mbs,
-                                         nrhs, lo_plane(PREC, n_freq, N_d, ldm));
+    if (sm > (size_t)kFftSmemMax) return cudaErrorInvalidValue;
+    k_gemv_adj<PREC, NB, kGemvThreads, kAdjUnroll><<<grid, kGemvThreads, sm, st>>>(
+        static_cast<const typename S::elem*>(fhat), scales, N_d, N_m, ldm, static_cast<const V*>(dh), dbs,
+        static_cast<V*>(mh), mbs, nrhs, lo_plane(PREC, n_freq, N_d, ldm));
     count_launch();
     return cudaGetLastError();
+}
+
+// Every CTA's limit, once per context (as in prepare_gemv_multi).
+cudaError_t prepare_gemv()
+{
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto k) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmemMax);
+    };
+    set(k_gemv_adj<P_F32, 1, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_F32, 2, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_F64, 1, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_F16S, 1, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_BF16, 1, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_BF16, 2, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_BF16X2, 1, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_FP8S, 1, kGemvThreads, kAdjUnroll>);
+    return e;
 }
 
 cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int n_freq, int N_d,

@@ -25,6 +25,8 @@
 // F* sums along s, F per lane along l and then over the lanes in the tree of
 // the single-vector kernels: a vector's result does not depend on its batch,
 // except where warps share the blocks along l (few rows or few frequencies).
+#include <utility>
+
 #include "gemv_store.cuh"
 
 namespace btt {
@@ -77,6 +79,7 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes)
 // read: two would need 128 bytes per clock at the full FP32 rate, all the
 // shared pipe has.
 constexpr int kFwdRows = 4, kFwdWarps = 8, kFwdChunk = 512;
+constexpr int kFwdSmemMax = 64 * 1024;   // set by prepare_gemv_multi
 
 // Whether two blocks' raw units fit beside the accumulators in 128 registers,
 // and whether 80 registers (three CTAs of 8 warps per SM) hold the kernel.
@@ -398,7 +401,7 @@ static cudaError_t fwd_multi(const void* fhat, const float* scales, int n_freq, 
     tiles = (groups + rg - 1) / rg;
     int wk = kFwdWarps / rg;
     int ch = kFwdChunk;
-    while (ch / BLK < wk && (size_t)2 * NB * ch * 2 * sizeof(float2) <= 64 * 1024) ch *= 2;
+    while (ch / BLK < wk && (size_t)2 * NB * ch * 2 * sizeof(float2) <= (size_t)kFwdSmemMax) ch *= 2;
     if (wk > ch / BLK) wk = ch / BLK;
     if (wk > nblk) wk = nblk;
     int its_log2 = 0;   // blocks per chunk
@@ -407,15 +410,10 @@ static cudaError_t fwd_multi(const void* fhat, const float* scales, int n_freq, 
     const size_t need = (size_t)rg * wk * kFwdRows * NB * 2 * sizeof(float);
     size_t sm = (size_t)2 * NB * ch * sizeof(float2);
     if (sm < need) sm = need;
-    auto kern = k_gemv_fwd_multi<PREC, NB>;
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-    }
     dim3 grid((nrhs + per - 1) / per, tiles, n_freq);
-    kern<<<grid, rg * wk * 32, sm, st>>>(static_cast<const typename S::elem*>(fhat), scales, N_d, ldm,
-                                         static_cast<const float2*>(xh), xbs, static_cast<float2*>(dh), dbs, nrhs,
-                                         per, rg, wk, ch, its_log2, lo_plane(PREC, n_freq, N_d, ldm));
+    k_gemv_fwd_multi<PREC, NB><<<grid, rg * wk * 32, sm, st>>>(
+        static_cast<const typename S::elem*>(fhat), scales, N_d, ldm, static_cast<const float2*>(xh), xbs,
+        static_cast<float2*>(dh), dbs, nrhs, per, rg, wk, ch, its_log2, lo_plane(PREC, n_freq, N_d, ldm));
     count_launch();
     return cudaGetLastError();
 }
@@ -497,6 +495,30 @@ static cudaError_t adj_groups(const void* fhat, const float* scales, int n_freq,
     }
 #undef BTT_ADJ
     return cudaErrorInvalidValue;
+}
+
+template <int PREC, int... NB> static cudaError_t fwd_limits(std::integer_sequence<int, NB...>)
+{
+    cudaError_t e = cudaSuccess;
+    ((e = e != cudaSuccess ? e
+                           : cudaFuncSetAttribute(k_gemv_fwd_multi<PREC, NB>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmemMax)),
+     ...);
+    return e;
+}
+
+// The largest a launch may ask for, once per context: the limit belongs to
+// the kernel, so one set per launch to that launch's size may be lowered by
+// another thread's launch before the first has been made.
+cudaError_t prepare_gemv_multi()
+{
+    using Groups = std::integer_sequence<int, 2, 3, 4, 5, 6, 7, 8>;
+    cudaError_t e = fwd_limits<P_F32>(Groups{});
+    if (e == cudaSuccess) e = fwd_limits<P_F16S>(Groups{});
+    if (e == cudaSuccess) e = fwd_limits<P_BF16>(Groups{});
+    if (e == cudaSuccess) e = fwd_limits<P_BF16X2>(std::integer_sequence<int, 2, 3>{});
+    if (e == cudaSuccess) e = fwd_limits<P_FP8S>(Groups{});
+    return e;
 }
 
 cudaError_t launch_gemv_fwd_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int ldm,

@@ -140,6 +140,7 @@ bool pf_hess_mid(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* 
                  const double2* tw, cudaStream_t st, cudaError_t* err);
 
 // ---- per-frequency products (gemv_kernels.cu) ----
+cudaError_t prepare_gemv();
 // dh[b][w][s] = sum_l Fhat[w][s][l] xh[b][w][l]          (Alg. 2, apply_matrix)
 cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
                             int ldm, const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs,
@@ -150,6 +151,7 @@ cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int
                             int nrhs, cudaStream_t st);
 
 // Both for several vectors at once, FP32 formats (gemv_multi.cu).
+cudaError_t prepare_gemv_multi();
 cudaError_t launch_gemv_fwd_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int ldm,
                                   const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs, cudaStream_t st);
 cudaError_t launch_gemv_adj_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int N_m,

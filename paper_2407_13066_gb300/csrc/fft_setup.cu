@@ -230,11 +230,14 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
                 d = make_double2(z.y + zc.y, zc.x - z.x);
             }
             if ((PREC == P_F16S || PREC == P_FP8S) && find_max) {
-                // the lanes of a row first, then one shared maximum per row
-                double m = one && w <= N ? fmax(fabs(a.x), fabs(a.y)) : 0.;
-                if (both && w <= N) m = fmax(m, fmax(fabs(d.x), fabs(d.y)));
-                for (int o = Wc / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (c == 0 && w <= N) atomicMax(&smax[w], (unsigned long long)__double_as_longlong(m));
+                // the lanes of a row first, then one shared maximum per row;
+                // as bits, in the order of the magnitudes with NaN on top: an
+                // entry without a finite part leaves the slice at scale 1
+                auto bits = [](double2 z) { return (unsigned long long)__double_as_longlong(fmax(fabs(z.x), fabs(z.y))); };
+                unsigned long long m = one && w <= N ? bits(a) : 0ull;
+                if (both && w <= N) m = max(m, bits(d));
+                for (int o = Wc / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (c == 0 && w <= N) atomicMax(&smax[w], m);
                 continue;
             }
             if (w > N || !one) continue;

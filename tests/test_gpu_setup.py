@@ -60,3 +60,18 @@ def test_fp64_vectors(shape):
         assert rel(op.adjoint(dev(d)), fft_method.adjoint(Fh, d)) < 1e-12
         assert rel(op.hessian(dev(m), dev(g)), fft_method.adjoint(Fh, g * f)) < 1e-12
         assert rel(op.hessian(dev(m)), fft_method.adjoint(Fh, f)) < 1e-12
+
+
+@pytest.mark.parametrize("prec", ["f16s", "fp8s"])
+@pytest.mark.parametrize("shape", [(16, 4, 6), (360, 2, 9), (6480, 1, 3)])
+def test_scales_of_a_slice_that_holds_nan(shape, prec):
+    """Two NaN samples in neighbouring columns make both columns NaN at every
+    frequency; such a slice has no largest magnitude and takes scale 1, from
+    the prime-factor kernel as from the mixed-radix one (6480)."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("setupnan", N_t, N_d, N_m, tau=N_t / 5, seed=N_t)
+    F = synth.blocks(w)
+    F[N_t // 3, 0, 0:2] = np.nan
+    with btt.Operator(F, precision=prec) as op:
+        _, sc = op.copy_fhat()
+    np.testing.assert_array_equal(sc, np.ones(N_t + 1))

@@ -455,6 +455,22 @@ static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
     return nrhs > 4 || ldm >= 4096 || N_d <= 16;
 }
 
+// FP64 F on two warps per CTA in place of eight: the sums over lanes cost as
+// much as 18 columns per warp, so short rows gain (1000 x 100 x 1000 824 -> 731
+// us, 5000 x 10 x 200 183 -> 134) while enough CTAs keep the SMs busy.  Time on
+// two warps over eight, by CTAs and row length:
+//   CTAs             128   512    1000       1400       2000       4000       8192
+//   up to 152       ~1.0   1.5    1.6        1.7        2.0        2.1        2.7
+//   153 .. 304       0.9   0.9  1.0-1.15   1.0-1.25   1.0-1.26   1.1-2.3    1.1-2.5
+//   305 .. 608       0.7   0.8    0.9        0.9      0.9-1.26   1.0-1.6    1.0-1.7
+//   above 608        0.6   0.8    0.9        0.95       1.0        1.0        1.05
+// The number of vectors has no part in it: a vector's sums keep their order.
+static bool f64_two_warps(int n_freq, int N_d, int ldm)
+{
+    const int64_t ctas = (int64_t)n_freq * ((N_d + 3) / 4);
+    return ctas > 304 ? ldm <= 1400 : (ctas > 152 && ldm <= 512);
+}
+
 cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
                             int ldm, const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs,
                             cudaStream_t st)
@@ -465,12 +481,9 @@ cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int
     switch (prec) {
         case P_F32: return fwd_dispatch<P_F32>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_F64:
-            // short rows on two warps: the sums over lanes cost as much as 18
-            // columns per warp (1000 x 100 x 1000 824 -> 731 us, 5000 x 10 x 200
-            // 183 -> 134)
-            return ldm <= 8192 ? fwd_launch<P_F64, 4, 1, 64>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st)
-                               : fwd_launch<P_F64, 4, 1, kGemvThreads>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs,
-                                                                       nrhs, st);
+            return f64_two_warps(n_freq, N_d, ldm)
+                       ? fwd_launch<P_F64, 4, 1, 64>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st)
+                       : fwd_launch<P_F64, 4, 1, kGemvThreads>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_F16S: return fwd_dispatch<P_F16S>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_BF16: return fwd_dispatch<P_BF16>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
         case P_BF16X2: return fwd_dispatch<P_BF16X2>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);

@@ -519,6 +519,7 @@ cudaError_t prepare_gemv()
     };
     set(k_gemv_adj<P_F32, 1, kGemvThreads, kAdjUnroll>);
     set(k_gemv_adj<P_F32, 2, kGemvThreads, kAdjUnroll>);
+    set(k_gemv_adj<P_F32, 4, kGemvThreads, kAdjUnroll>);
     set(k_gemv_adj<P_F64, 1, kGemvThreads, kAdjUnroll>);
     set(k_gemv_adj<P_F16S, 1, kGemvThreads, kAdjUnroll>);
     set(k_gemv_adj<P_BF16, 1, kGemvThreads, kAdjUnroll>);
@@ -534,12 +535,16 @@ cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int
 {
     if (nrhs <= 0) return cudaSuccess;
     // several vectors: the group kernel (two in FP32 and BF16 stay here: 592
-    // against 602 us at 256 x 200 x 10000, 155 against 177 at 1500 x 24 x 6000)
+    // against 602 us at 256 x 200 x 10000, 155 against 177 at 1500 x 24 x 6000;
+    // and 3-4 in FP32 on at most 3 rows, its unrolled loop's remainder: 3355 x 1 x
+    // 1914 52 against 70 us, 8937 x 2 x 310 29 against 41)
     // (column tiles of at least 256 index grid.y)
-    if (prec != P_F64 && nrhs > (prec == P_BF16 || prec == P_F32 ? 2 : 1) && ldm <= 256 * 65535)
+    const int here = prec == P_F32 ? (N_d <= 3 ? 4 : 2) : (prec == P_BF16 ? 2 : 1);
+    if (prec != P_F64 && nrhs > here && ldm <= 256 * 65535)
         return launch_gemv_adj_multi(prec, fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
     switch (prec) {
         case P_F32:
+            if (nrhs > 2) return adj_launch<P_F32, 4>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
             return nrhs == 1 ? adj_launch<P_F32, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st)
                              : adj_launch<P_F32, 2>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);
         case P_F64: return adj_launch<P_F64, 1>(fhat, scales, n_freq, N_d, N_m, ldm, dh, dbs, mh, mbs, nrhs, st);

@@ -730,7 +730,11 @@ static size_t smem_of(const FftGeom& g, int C, int wql)
 //   1500: 4 CTAs 16 columns 620 / 835; 2 CTAs 8 644 / 785, 16 664 / 864
 //   9000: 8 CTAs 8 columns (87 KB) 932 / 1356, 4 (52 KB) 1129 / 1458,
 //         16 (157 KB, one CTA per SM) 1190 / 2237; 4 CTAs 4 (100 KB) 1446 / 1306
-// Few columns take narrower tiles, so that two CTAs per SM have work.
+// Few columns take narrower tiles, so that two CTAs per SM have work, but no
+// more CTAs than are resident at once: a second wave of small ones cost more
+// than the idle SMs (us, input / inverse, unbounded -> so: 12 steps, 2000
+// columns 8.2 / 8.7 -> 6.2 / 6.2; 420 steps 13.0 / 14.4 -> 10.3 / 10.3; 1500 steps, 16
+// x 30 columns 19.1 / 21.5 -> 12.4 / 14.4).
 static bool pick(const FftGeom& g, int ncols, int nb, Shape* s)
 {
     if (!g.res_tab) return false;
@@ -750,7 +754,12 @@ static bool pick(const FftGeom& g, int ncols, int nb, Shape* s)
         }
     }
     if (best < 0) return false;
-    while (s->wql > 0 && (int64_t)s->C * nb * ((ncols + (4 << s->wql) - 1) / (4 << s->wql)) < 2 * 152) --s->wql;
+    auto ctas = [&](int w) { return (int64_t)s->C * nb * ((ncols + (4 << w) - 1) / (4 << w)); };
+    auto resident = [&](int w) {
+        const size_t sm = smem_of(g, s->C, w);
+        return 152 * (sm <= 76 * 1024 ? 3 : sm <= 113 * 1024 ? 2 : 1);
+    };
+    while (s->wql > 0 && ctas(s->wql) < 2 * 152 && ctas(s->wql - 1) <= resident(s->wql - 1)) --s->wql;
     return true;
 }
 

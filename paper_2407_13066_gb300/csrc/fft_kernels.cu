@@ -449,7 +449,7 @@ cudaError_t launch_hess_mid(cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols, c
         // one launch of the kernel below wins, 14.4 against 10.5 us at 5; it
         // also sums g (F m)^2 for the CG solver)
         const int64_t n = (int64_t)g.N_t * ncols;
-        if (!part && scratch && g.N_t >= 100 &&
+        if (!part && scratch && res_mid(g, ncols) &&
             res_irfft(X, ldx, bsx, ncols, scratch, ncols, n, gam, nb, g, tw, st, nullptr, &e)) {
             if (e != cudaSuccess) return e;
             res_rfft(scratch, ncols, n, ncols, X, ldx, bsx, nb, g, tw, st, nullptr, &e);

@@ -49,7 +49,9 @@ using fq::f2;
 using fq::fma;
 using fq::mul;
 
-constexpr int NT = 256;
+// Threads per CTA (threads_of); 24 warps per SM with 3, 2 or 1 CTAs.
+constexpr int kNT = 256, kNTLong = 384, kNTLongest = 768;
+constexpr int ctas_per_sm(int nt) { return nt == kNT ? 3 : nt == kNTLong ? 2 : 1; }
 // Radices up to 10 run in 80 registers, three CTAs per SM; up to 16 they take
 // 128 (two CTAs), and the passes saved do not make up for the latency left
 // uncovered (N_t = 1500, 8 columns on 2 CTAs: 866 / 1147 us against 646 / 911).
@@ -189,7 +191,7 @@ __device__ __forceinline__ ulonglong2 quad(float2 w) { return make_ulonglong2(fq
 
 // One in-place pass over the CTA's 2 M positions: radix R on sub-blocks of Mp
 // (forward: DFT, then twiddles; inverse: conjugate twiddles, then DFT).
-template <int R, bool INV>
+template <int NT, int R, bool INV>
 __device__ __forceinline__ void pass(ulonglong2* buf, int total, int Mp, unsigned magic, int wql, int tstep,
                                      const float2* tws)
 {
@@ -217,26 +219,26 @@ __device__ __forceinline__ void pass(ulonglong2* buf, int total, int Mp, unsigne
     __syncthreads();
 }
 
-template <bool INV>
+template <int NT, bool INV>
 __device__ __forceinline__ void radix_pass(int R, ulonglong2* buf, int total, int Mp, unsigned magic, int wql,
                                            int tstep, const float2* tws)
 {
     switch (R) {
-        case 2: pass<2, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 3: pass<3, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 4: pass<4, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 5: pass<5, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 6: pass<6, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 7: pass<7, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 8: pass<8, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        case 9: pass<9, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
-        default: pass<10, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 2: pass<NT, 2, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 3: pass<NT, 3, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 4: pass<NT, 4, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 5: pass<NT, 5, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 6: pass<NT, 6, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 7: pass<NT, 7, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 8: pass<NT, 8, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        case 9: pass<NT, 9, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
+        default: pass<NT, 10, INV>(buf, total, Mp, magic, wql, tstep, tws); break;
     }
 }
 
 // Shared memory of a CTA: the tile [2 M][Wq] quads, the M-point twiddles and
 // the position table (position of a frequency).
-struct Smem {
+template <int NT> struct Smem {
     ulonglong2* buf;
     float2* tws;
     unsigned short* pos;
@@ -393,14 +395,14 @@ __device__ __forceinline__ cq swap_half(cq v)
     return {{__shfl_xor_sync(0xffffffffu, v.re.u, 1)}, {__shfl_xor_sync(0xffffffffu, v.im.u, 1)}};
 }
 
-template <int C, class Out>
-__global__ void __launch_bounds__(NT, 3)
+template <int C, class Out, int NT>
+__global__ void __launch_bounds__(NT, ctas_per_sm(NT))
 k_rfft_res(const float* __restrict__ x, int64_t ldx, int64_t bsx, int ncols, Out out, ResPlan plan, int wql,
            const float2* __restrict__ tw, const int* __restrict__ tab, const float* const* __restrict__ xptr)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int S = 2 * C;
-    Smem sm_(smem_raw, plan.M, wql);
+    Smem<NT> sm_(smem_raw, plan.M, wql);
     ulonglong2* buf = sm_.buf;
     const int M = plan.M, L = S * M, N = C * M, wm = (1 << wql) - 1;
     const int r = C == 1 ? 0 : cta_rank();
@@ -490,7 +492,7 @@ k_rfft_res(const float* __restrict__ x, int64_t ldx, int64_t bsx, int ncols, Out
 
     int Mp = M, tstep = 1;
     for (int p = 0; p < plan.np; ++p) {
-        radix_pass<false>(plan.radix[p], buf, 2 * M, Mp, plan.magic[p], wql, tstep, sm_.tws);
+        radix_pass<NT, false>(plan.radix[p], buf, 2 * M, Mp, plan.magic[p], wql, tstep, sm_.tws);
         Mp /= plan.radix[p];
         tstep *= plan.radix[p];
     }
@@ -541,15 +543,15 @@ __device__ __forceinline__ cq load_spectra(const __nv_bfloat162* __restrict__ ro
     return {fq::pack(a.x, d.x), fq::pack(a.y, d.y)};
 }
 
-template <int C, class TX>
-__global__ void __launch_bounds__(NT, 3)
+template <int C, class TX, int NT>
+__global__ void __launch_bounds__(NT, ctas_per_sm(NT))
 k_irfft_res(const TX* __restrict__ X, int64_t ldx, int64_t bsx, int ncols, float* __restrict__ y, int64_t ldy,
             int64_t bsy, const float* __restrict__ gam, ResPlan plan, int wql, const float2* __restrict__ tw,
             const int* __restrict__ tab, float* const* __restrict__ yptr)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int S = 2 * C;
-    Smem sm_(smem_raw, plan.M, wql);
+    Smem<NT> sm_(smem_raw, plan.M, wql);
     ulonglong2* buf = sm_.buf;
     const int M = plan.M, L = S * M, N = C * M, wm = (1 << wql) - 1;
     const int r = C == 1 ? 0 : cta_rank();
@@ -598,7 +600,7 @@ k_irfft_res(const TX* __restrict__ X, int64_t ldx, int64_t bsx, int ncols, float
     for (int p = plan.np - 1; p >= 0; --p) {
         Mp *= plan.radix[p];
         tstep /= plan.radix[p];
-        radix_pass<true>(plan.radix[p], buf, 2 * M, Mp, plan.magic[p], wql, tstep, sm_.tws);
+        radix_pass<NT, true>(plan.radix[p], buf, 2 * M, Mp, plan.magic[p], wql, tstep, sm_.tws);
     }
 
     uint32_t src[C];
@@ -694,11 +696,11 @@ template <typename K> static cudaError_t set_smem(K k)
 }
 
 template <typename K, typename... A>
-static cudaError_t launch(K kern, int C, int tiles, int nb, size_t sm, cudaStream_t st, A... args)
+static cudaError_t launch(K kern, int C, int threads, int tiles, int nb, size_t sm, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(tiles * C), (unsigned)nb, 1);
-    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = sm;
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -715,10 +717,21 @@ struct Shape {
     int C, wql;
 };
 
+// Odd lengths above 2048 have no cluster to spread over, and their CTA leaves
+// room for one other on its SM or for none: with 8 warps each the latency of
+// a pass was left uncovered.  Inverse, us, the kernels of fft_kernels.cu / 8 warps
+// / now: 3125 steps, 8 x 1200 columns 450 / 497 / 365, 30 columns 18 / 25 / 23; 2187 steps
+// (two CTAs), 8 x 800 columns 263 / 147 / 135.
+static int threads_of(const FftGeom& g, int C)
+{
+    if (C > 1 || g.N_t <= 2048) return kNT;
+    return (size_t)g.N_t * 42 + kNTLong * 16 <= 113 * 1024 ? kNTLong : kNTLongest;
+}
+
 static size_t smem_of(const FftGeom& g, int C, int wql)
 {
     const size_t M = g.N_t / C;
-    return ((2 * M) << wql) * 16 + NT * 16 + M * 10;
+    return ((2 * M) << wql) * 16 + threads_of(g, C) * 16 + M * 10;
 }
 
 // Cluster size and tile width.  Wide rows want few CTAs' worth of shared
@@ -847,37 +860,43 @@ cudaError_t prepare_res_fft()
     auto set = [&](auto k) {
         if (e == cudaSuccess) e = res::set_smem(k);
     };
-    set(res::k_rfft_res<1, res::OutC64>);
-    set(res::k_rfft_res<2, res::OutC64>);
-    set(res::k_rfft_res<4, res::OutC64>);
-    set(res::k_rfft_res<8, res::OutC64>);
-    set(res::k_rfft_res<1, res::OutStack>);
-    set(res::k_rfft_res<2, res::OutStack>);
-    set(res::k_rfft_res<4, res::OutStack>);
-    set(res::k_rfft_res<8, res::OutStack>);
-    set(res::k_irfft_res<1, float2>);
-    set(res::k_irfft_res<2, float2>);
-    set(res::k_irfft_res<4, float2>);
-    set(res::k_irfft_res<8, float2>);
-    set(res::k_irfft_res<1, __nv_bfloat162>);
-    set(res::k_irfft_res<2, __nv_bfloat162>);
-    set(res::k_irfft_res<4, __nv_bfloat162>);
-    set(res::k_irfft_res<8, __nv_bfloat162>);
+    auto all = [&](auto c) {
+        constexpr int C = decltype(c)::value;
+        set(res::k_rfft_res<C, res::OutC64, res::kNT>);
+        set(res::k_rfft_res<C, res::OutStack, res::kNT>);
+        set(res::k_irfft_res<C, float2, res::kNT>);
+        set(res::k_irfft_res<C, __nv_bfloat162, res::kNT>);
+    };
+    all(std::integral_constant<int, 1>{});
+    all(std::integral_constant<int, 2>{});
+    all(std::integral_constant<int, 4>{});
+    all(std::integral_constant<int, 8>{});
+    auto wide = [&](auto nt) {
+        constexpr int NT = decltype(nt)::value;
+        set(res::k_rfft_res<1, res::OutC64, NT>);
+        set(res::k_rfft_res<1, res::OutStack, NT>);
+        set(res::k_irfft_res<1, float2, NT>);
+        set(res::k_irfft_res<1, __nv_bfloat162, NT>);
+    };
+    wide(std::integral_constant<int, res::kNTLong>{});
+    wide(std::integral_constant<int, res::kNTLongest>{});
     return e;
 }
 
-// Dispatch on the cluster size.
-#define BTT_RES(K, T, ...)                                                                             \
-    (s.C == 1   ? res::launch(res::K<1, T>, 1, tiles, nb, sm, st, __VA_ARGS__)                         \
-     : s.C == 2 ? res::launch(res::K<2, T>, 2, tiles, nb, sm, st, __VA_ARGS__)                         \
-     : s.C == 4 ? res::launch(res::K<4, T>, 4, tiles, nb, sm, st, __VA_ARGS__)                         \
-                : res::launch(res::K<8, T>, 8, tiles, nb, sm, st, __VA_ARGS__))
+// Dispatch on the cluster size and the threads per CTA.
+#define BTT_RES(K, T, ...)                                                                                      \
+    (nt == res::kNTLongest ? res::launch(res::K<1, T, res::kNTLongest>, 1, nt, tiles, nb, sm, st, __VA_ARGS__)  \
+     : nt == res::kNTLong  ? res::launch(res::K<1, T, res::kNTLong>, 1, nt, tiles, nb, sm, st, __VA_ARGS__)     \
+     : s.C == 1            ? res::launch(res::K<1, T, res::kNT>, 1, nt, tiles, nb, sm, st, __VA_ARGS__)         \
+     : s.C == 2            ? res::launch(res::K<2, T, res::kNT>, 2, nt, tiles, nb, sm, st, __VA_ARGS__)         \
+     : s.C == 4            ? res::launch(res::K<4, T, res::kNT>, 4, nt, tiles, nb, sm, st, __VA_ARGS__)         \
+                           : res::launch(res::K<8, T, res::kNT>, 8, nt, tiles, nb, sm, st, __VA_ARGS__))
 #define BTT_RES_SETUP                                                       \
     res::Shape s;                                                           \
     if (!res::pick(g, ncols, nb, &s)) return false;                         \
     const ResPlan& plan = g.res[res::lg(s.C)];                              \
-    const int tiles = res::tiles_of(ncols, s);                              \
-    const size_t sm = res::smem_of(g, s.C, s.wql);                                   \
+    const int tiles = res::tiles_of(ncols, s), nt = res::threads_of(g, s.C); \
+    const size_t sm = res::smem_of(g, s.C, s.wql);                          \
     const int* tab = g.res_tab + plan.tab
 
 bool res_rfft(const float* x, int64_t ldx, int64_t bsx, int ncols, float2* X, int64_t ldo, int64_t bso, int nb,
@@ -903,9 +922,24 @@ bool res_irfft(const float2* X, int64_t ldx, int64_t bsx, int ncols, float* y, i
                const float* gam, int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr,
                cudaError_t* err)
 {
+    // Few columns of a long odd length, one CTA's latency: the mixed-radix
+    // kernel's is shorter (30 columns, this one / that: 3125 23 / 19 us, 4375
+    // 27 / 23, 5145 32 / 25; below 3000 steps they are level).  The number of
+    // vectors has no part in it: a vector's result stays the same.
+    if (g.N_t % 2 && g.N_t > 3000 && ncols <= 32) return false;
     BTT_RES_SETUP;
     *err = BTT_RES(k_irfft_res, float2, X, ldx, bsx, ncols, y, ldy, bsy, gam, plan, s.wql, tw, tab, yptr);
     return true;
+}
+
+// Odd lengths above 2048 (no cluster) take two launches of 20-30 us where the
+// columns are few; one launch of the mixed-radix kernel is shorter (us, two
+// launches / one; 30 columns, 1 and 8 vectors, then 100 columns and 8):
+//   2401  33 / 29  35 / 29  57 / 62     3125  43 / 35  43 / 35  80 / 80
+//   4375  55 / 43  55 / 43  102 / 103   5145  68 / 47  68 / 48  131 / 115
+bool res_mid(const FftGeom& g, int ncols)
+{
+    return g.N_t >= 100 && !(g.N_t % 2 && g.N_t > 2048 && ncols <= (g.N_t > 4200 ? 100 : 32));
 }
 
 bool res_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy, int64_t bsy,

@@ -213,6 +213,8 @@ bool res_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols
 // True when 2 N_t has a fixed radix plan.
 bool static_plan(const FftGeom& g);
 // Its fixed-plan form; false for lengths without a fixed plan.
+// Whether res_irfft and res_rfft are the faster middle step for ncols columns.
+bool res_mid(const FftGeom& g, int ncols);
 bool static_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy,
                        int64_t bsy, int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr,
                        cudaError_t* err);

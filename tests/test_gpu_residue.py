@@ -76,3 +76,43 @@ def test_pointer_table(N_t):
             got = raw_out[b][1:n + 1].double().cpu().numpy().reshape(N_t, N_m)
             np.testing.assert_array_equal(got, ref[b])
             assert raw_out[b][0] == 0 and float(raw_out[b][n + 1:].abs().sum()) == 0
+
+
+LONG_ODD = [  # (N_t, N_d, N_m): 384 threads per CTA to 2601 steps, 768 above; up to 32 columns the mixed-radix kernels
+    (2187, 3, 37), (2401, 33, 6), (2625, 2, 40), (2835, 1, 33), (3125, 2, 36), (3375, 34, 2), (4375, 2, 101),
+    (5145, 101, 3), (3125, 1, 20), (5103, 2, 8),
+]
+
+
+@pytest.mark.parametrize("shape", LONG_ODD)
+def test_long_odd_lengths(shape):
+    """One CTA per tile at its largest sizes, against the oracle's FFT
+    algorithm; a vector's bits are the same alone and in a batch of five."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("resodd", N_t, N_d, N_m, tau=N_t / 5, seed=N_t + N_m)
+    F, m, d, g = inputs(w, nrhs=5)
+    Fh = fft_method.setup(F)
+    with btt.Operator(torch.from_numpy(F).cuda(), precision="f32", max_nrhs=5) as op:
+        m, d, g = (dev(a, torch.float32) for a in (m, d, g))
+        for f, x, ref in ((op.matvec, m, fft_method.forward(Fh, host(m))),
+                          (op.adjoint, d, fft_method.adjoint(Fh, host(d))),
+                          (lambda v: op.hessian(v, g), m,
+                           fft_method.adjoint(Fh, host(g) * fft_method.forward(Fh, host(m))))):
+            y = f(x)
+            assert rel(host(y), ref) < TOL["f32"]
+            assert torch.equal(torch.cat([f(x[j:j + 1]) for j in range(5)]), y)
+        op.device_status()
+
+
+@pytest.mark.parametrize("prec", ["bf16", "bf16x2"])
+@pytest.mark.parametrize("shape", [(2401, 3, 19), (3125, 2, 35), (5145, 1, 6)])
+def test_long_odd_tensor_operands(shape, prec):
+    """Their BF16 forms, to the oracle at the format's tolerance."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("resoddtc", N_t, N_d, N_m, tau=N_t / 5, seed=N_t + 3 * N_m)
+    F, m, d, _ = inputs(w, nrhs=17)
+    Fh = fft_method.setup(F)
+    with btt.Operator(torch.from_numpy(F).cuda(), precision=prec, max_nrhs=17, gemm="tensor") as op:
+        assert rel(host(op.matvec(dev(m, torch.float32))), fft_method.forward(Fh, m)) < TOL[prec]
+        assert rel(host(op.adjoint(dev(d, torch.float32))), fft_method.adjoint(Fh, d)) < TOL[prec]
+        op.device_status()

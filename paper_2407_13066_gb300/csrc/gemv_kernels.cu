@@ -437,22 +437,35 @@ static cudaError_t fwd_dispatch(const void* fhat, const float* scales, int n_fre
     return rows_shape<PREC, 4, U4, 512>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
 }
 
-// Where the group kernel of gemv_multi.cu is the faster one for F.  Measured
-// (this file's kernel -> the group kernel, us per launch):
-//   256 x 200 x 10000: FP32 3 vectors 779 -> 661, 8 1513 -> 1004, 32 5890 ->
-//     3807; FP8 3 vectors 1007 -> 423; 2 vectors within 5% or slower (FP32
-//     608 -> 642); split pairs (16 more registers per row) 4 876 -> 1111;
-//   300 x 37 x 3001, a CTA's rows too short for its staging: FP32 4 vectors
-//     63 -> 75, 8 123 -> 102;
-//   64 x 8 x 20000, 65 CTAs of 20 rows here: FP32 2 vectors 64 -> 35, split
-//     pairs 123 -> 31 (l split over warps), but FP16 32 vectors 170 -> 281.
+// Where the group kernel of gemv_multi.cu is the faster one for F (one warp
+// per row in both, the same sums in the same order).  Time there over time here
+// by row groups of 4 in the launch, blocks per row (32 lanes x 16 bytes) and
+// vectors; means over 130 shapes of 6-9000 frequencies, 1-500 rows and 20-20000
+// columns:
+//   row groups            153-304  305-608  609-1216  1217-2432  2433-4864   above
+//   FP32  3 - 4, short      1.01     1.13     1.07       0.88       0.85      0.72
+//               long         -       1.15   0.8-0.97   0.70-0.87
+//         5 - 8, short      1.05     1.01     0.86       0.73       0.65      0.53
+//               long         -       1.2    0.52-0.70  0.51-0.85
+//         16 - 32           0.79     0.78     0.74       0.67       0.61      0.53
+//   BF16  3 - 4, short      1.12     1.21     1.04       0.97       0.93      0.89
+//               long        1.02   0.94-1.05 0.69-1.07  0.63-0.80
+//         5 - 8, short      1.24     1.20     0.96       0.90       0.80      0.67
+//               long        1.07   0.85-1.0  0.54-0.89  0.57-0.91
+//   FP8   3 - 8, short      1.05     1.02     0.92       0.80       0.68      0.70
+//               long        0.7    0.46-0.63 0.39-0.89  0.57-0.76
+// (long: more than 12 blocks; BF16 3 - 4 on 305-608 groups 1.05 up to 40 blocks,
+// 0.94 and below beyond.)  Two vectors: mixed (BF16 0.9-1.4, FP32 0.8-1.4);
+// split pairs (16 more registers per row) 0.9-1.4, by whether groups of three
+// divide the batch.
 static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
 {
-    if (nrhs < 2 || N_d > 32 * 65535) return false;   // (row tiles index grid.y)
-    if (nrhs > 16 && N_d <= 8 && prec != P_F32) return false;
-    if ((int64_t)n_freq * ((N_d + 19) / 20) < 152) return true;
-    if (nrhs == 2 || prec == P_BF16X2) return false;
-    return nrhs > 4 || ldm >= 4096 || N_d <= 16;
+    if (nrhs < 3 || prec == P_BF16X2 || N_d > 32 * 65535) return false;   // (row tiles index grid.y)
+    const int64_t groups = (int64_t)n_freq * ((N_d + 3) / 4);
+    const bool few = nrhs <= 4, wide = ldm > 12 * (prec == P_F32 ? 64 : prec == P_FP8S ? 256 : 128);
+    if (prec == P_F32) return groups > (few ? (wide ? 608 : 1216) : nrhs <= 12 ? 608 : 304);
+    if (prec == P_FP8S) return wide || groups > 608;
+    return groups > (wide ? (few && ldm <= 40 * 128 ? 608 : 304) : (few ? 1216 : 608));
 }
 
 // FP64 F on two warps per CTA in place of eight: the sums over lanes cost as
@@ -476,7 +489,7 @@ cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int
                             cudaStream_t st)
 {
     if (nrhs <= 0) return cudaSuccess;
-    if (prec != P_F64 && fwd_multi_wins(prec, n_freq, N_d, ldm, nrhs))
+    if (prec != P_F64 && (fwd_slices(prec, n_freq, N_d, ldm) > 1 || fwd_multi_wins(prec, n_freq, N_d, ldm, nrhs)))
         return launch_gemv_fwd_multi(prec, fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);
     switch (prec) {
         case P_F32: return fwd_dispatch<P_F32>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, st);

@@ -1,9 +1,13 @@
 // Per-frequency products for several right-hand sides on the FP32 units:
 //     F :  dhat_n[w][s] = sum_l Fhat[w][s][l] xhat_n[w][l]
 //     F*:  mhat_n[w][l] = sum_s conj(Fhat[w][s][l]) dhat_n[w][s]
-// for groups of up to 8 vectors n that share one pass over Fhat.  At NB
-// vectors a complex64 entry (8 bytes) feeds 8 NB flops, so the bound moves
-// from HBM (NB <= 4) to the FP32 units (128 lanes per SM and clock) at 8.
+// for groups of up to 8 vectors n that share one pass over Fhat.  An entry
+// feeds 8 flops per vector: at 256 x 200 x 10000 and 8 vectors 0.44 ms of FP32
+// time (128 lanes per SM and clock) against 0.61 ms of HBM time for complex64,
+// 0.30 for the 4-byte formats and 0.15 for FP8, so the floor is HBM's in FP32
+// (up to 11 vectors) and the FP32 units' in the others (from 6 and 3 vectors
+// on).  What the kernels are bound by there is issue and latency (issue active
+// 63-68%, FMA pipe 47-51%).
 // Both kernels spare what stands beside the multiply-adds: a value read from
 // shared memory serves four rows (F) or a 16-byte unit of columns (F*).  The
 // arithmetic is scalar: paired f32x2 instructions need each Fhat value
@@ -23,8 +27,8 @@
 //   FP8   F  8 vectors 1997 -> 905;   F* 8 vectors 800 -> 726
 //
 // F* sums along s, F per lane along l and then over the lanes in the tree of
-// the single-vector kernels: a vector's result does not depend on its batch,
-// except where warps share the blocks along l (few rows or few frequencies).
+// the single-vector kernels; where warps share a row (fwd_slices) every F of the
+// operator does.  A vector's result does not depend on the batch it is in.
 #include <utility>
 
 #include "gemv_store.cuh"
@@ -67,8 +71,9 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes)
 }
 
 // ------------------------------------------------------------ F (Alg. 2)
-// CTA = rg warps x 4 rows of one frequency (times wk warps that share the
-// blocks along l when there are few rows) for a group of NB vectors; the
+// CTA = rg warps x 4 rows of one frequency (or 8 warps that share the blocks
+// of 4 rows, wk = 8, where rows and frequencies are few) for a group of NB
+// vectors; the
 // group is the fastest grid dimension, so CTAs sharing a Fhat tile run
 // together and repeats hit L2 (the kernel it replaces read Fhat twice from
 // HBM at 8 vectors).  A warp streams its rows with 16-byte loads, the next
@@ -78,8 +83,8 @@ __device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes)
 // read consecutive ones whatever the unit's width.  Four rows per value
 // read: two would need 128 bytes per clock at the full FP32 rate, all the
 // shared pipe has.
-constexpr int kFwdRows = 4, kFwdWarps = 8, kFwdChunk = 512;
-constexpr int kFwdSmemMax = 64 * 1024;   // set by prepare_gemv_multi
+constexpr int kFwdRows = 4, kFwdWarps = 8;
+constexpr int kFwdSmemMax = 128 * 1024;   // set by prepare_gemv_multi
 
 // Whether two blocks' raw units fit beside the accumulators in 128 registers,
 // and whether 80 registers (three CTAs of 8 warps per SM) hold the kernel.
@@ -89,7 +94,7 @@ template <int PREC, int NB> constexpr bool fwd_pipelined()
 }
 template <int PREC, int NB> constexpr int fwd_min_blocks()
 {
-    return NB == 2 && PREC != P_BF16X2 ? 3 : (NB == 3 && PREC == P_F32 ? 3 : 2);
+    return NB <= 2 && PREC != P_BF16X2 ? 3 : (NB == 3 && PREC == P_F32 ? 3 : 2);
 }
 
 template <int PREC, int NB>
@@ -278,7 +283,7 @@ template <int PREC, int NB> constexpr int adj_unroll()
 }
 template <int PREC, int NB> constexpr int adj_min_blocks()
 {
-    // 128 registers for 24 or more complex accumulators, 96 below
+    // 128 registers for 16 or more complex accumulators, 96 below
     return Store<PREC>::VPL * NB >= 16 ? 4 : 5;
 }
 
@@ -383,34 +388,58 @@ k_gemv_adj_multi(const typename Store<PREC>::elem* __restrict__ fhat, const floa
 }
 
 // ---------------------------------------------------------------- launchers
+// Warps that share a row of F along l (blocks g, g + 8, ... each): 1, or 8 where
+// rows and frequencies are few and the rows long, so that a warp's walk along
+// its row is what the launch waits for.  A function of the operator alone: the
+// order in which a row is summed must not depend on the batch a vector is in,
+// so in those shapes a single vector comes here as well.  Measured (us, one
+// warp per row in gemv_kernels.cu -> 8 here, 1 / 2 / 8 / 32 vectors):
+//   65 x 7 x 20000    FP32 35 / 61 / 113 / 150 -> 21 / 25 / 43 / 119, BF16 41 / 72 / 131 / 163 ->
+//                     17 / 28 / 60 / 197, split pairs 68 / 121 / 141 / 175 -> 21 / 29 / 81 / 265,
+//                     FP8 49 / 90 / 103 / 204 -> 15 / 23 / 62 / 196
+//   17 x 7 x 2500     FP32 6.3 / 8.3 / 10.5 / 10.5 -> 6.4 / 6.4 / 6.3 / 8.5, BF16 7.7 / 8.4 / 12.4 /
+//                     12.5 -> 6.3 / 8.2 / 8.2 / 12.5
+// Beyond these lines it loses (mean over 1 .. 32 vectors, time on 8 over the
+// better kernel of one warp): FP32 at 457-608 row groups up to 1.15, up to 12
+// blocks 1.0-1.15; 16-bit formats and pairs at 153-304 groups 1.06-1.2 up to 40
+// blocks, at 305-456 1.1-1.4; FP8 at 153-304 1.03-1.24.
+int fwd_slices(int prec, int n_freq, int N_d, int ldm)
+{
+    const int64_t groups = (int64_t)n_freq * ((N_d + kFwdRows - 1) / kFwdRows);
+    const int blk = prec == P_F32 ? 64 : (prec == P_FP8S ? 256 : 128), nblk = (ldm + blk - 1) / blk;
+    const bool yes = prec == P_F32    ? groups <= 456 && nblk > 12
+                     : prec == P_FP8S ? groups <= 152 && nblk > 12
+                                      : (groups <= 152 && nblk > 12) || (groups <= 304 && nblk > 40);
+    return yes ? kFwdWarps : 1;
+}
+
 template <int PREC, int NB>
 static cudaError_t fwd_multi(const void* fhat, const float* scales, int n_freq, int N_d, int ldm, const void* xh,
-                             int64_t xbs, void* dh, int64_t dbs, int nrhs, int per, cudaStream_t st)
+                             int64_t xbs, void* dh, int64_t dbs, int nrhs, int per, int wk, cudaStream_t st)
 {
     using S = Store<PREC>;
     constexpr int BLK = 32 * S::VPL;
     const int nblk = (ldm + BLK - 1) / BLK;
-    // Row groups of 4 spread evenly over tiles of at most 8 warps; with few
-    // rows, or too few tiles for the SMs, the spare warps share the blocks
-    // along l.
+    // Row groups of 4 spread evenly over tiles of at most 8 warps.
     const int groups = (N_d + kFwdRows - 1) / kFwdRows;
-    int tiles = (groups + kFwdWarps - 1) / kFwdWarps;
-    int rg = (groups + tiles - 1) / tiles;
     const int64_t vg = (nrhs + per - 1) / per;
-    while (rg > 1 && vg * n_freq * ((groups + rg - 1) / rg) < (PREC == P_F32 ? 4 : 2) * 152) rg = (rg + 1) / 2;
+    int tiles = (groups + kFwdWarps - 1) / kFwdWarps;
+    const int rg = wk > 1 ? 1 : (groups + tiles - 1) / tiles;
     tiles = (groups + rg - 1) / rg;
-    int wk = kFwdWarps / rg;
-    int ch = kFwdChunk;
-    while (ch / BLK < wk && (size_t)2 * NB * ch * 2 * sizeof(float2) <= (size_t)kFwdSmemMax) ch *= 2;
-    if (wk > ch / BLK) wk = ch / BLK;
-    if (wk > nblk) wk = nblk;
+    // Values per chunk: 512, less for CTAs of up to 4 warps, so that 16 warps of
+    // them fit (FP32) or one block (the formats that decode: few values arrive
+    // sooner than many; us at 512 / 256 / 128 values): 257 x 10 x 7648, BF16, 3
+    // vectors 50 / 48 / 45, 631 x 4 x 2923 25 / 25 / 23; FP32, 8 vectors, 2001 x 2 x
+    // 390 25 / 18 / 15.  A block for every warp that shares a row.
+    int ch = wk > 1 ? wk * BLK : rg > 4 || PREC == P_F32 ? 512 : BLK;
+    while (wk == 1 && ch > BLK && (size_t)2 * NB * ch * sizeof(float2) * (16 / rg) > 220 * 1024) ch /= 2;
     int its_log2 = 0;   // blocks per chunk
     while ((BLK << its_log2) < ch) ++its_log2;
     if (nblk * BLK < ch) ch = nblk * BLK;   // a single chunk
-    const size_t need = (size_t)rg * wk * kFwdRows * NB * 2 * sizeof(float);
+    const size_t need = wk > 1 ? (size_t)wk * kFwdRows * NB * 2 * sizeof(float) : 0;
     size_t sm = (size_t)2 * NB * ch * sizeof(float2);
     if (sm < need) sm = need;
-    dim3 grid((nrhs + per - 1) / per, tiles, n_freq);
+    dim3 grid((unsigned)vg, tiles, n_freq);
     k_gemv_fwd_multi<PREC, NB><<<grid, rg * wk * 32, sm, st>>>(
         static_cast<const typename S::elem*>(fhat), scales, N_d, ldm, static_cast<const float2*>(xh), xbs,
         static_cast<float2*>(dh), dbs, nrhs, per, rg, wk, ch, its_log2, lo_plane(PREC, n_freq, N_d, ldm));
@@ -455,11 +484,16 @@ template <int PREC>
 static cudaError_t fwd_groups(const void* fhat, const float* scales, int n_freq, int N_d, int ldm, const void* xh,
                               int64_t xbs, void* dh, int64_t dbs, int nrhs, cudaStream_t st)
 {
-    // (split pairs: a raw unit takes 8 registers, three vectors fill the rest)
-    const int64_t ctas = (int64_t)n_freq * ((N_d + kFwdRows * kFwdWarps - 1) / (kFwdRows * kFwdWarps));
-    const int per = group_size(nrhs, PREC == P_BF16X2 ? 3 : 8, ctas, 2);
+    const int wk = fwd_slices(PREC, n_freq, N_d, ldm), groups = (N_d + kFwdRows - 1) / kFwdRows;
+    // (split pairs: a raw unit takes 8 registers, three vectors fill the rest;
+    // 8 warps along a row: their chunk in 128 KB, one CTA per SM counted)
+    const int cap = PREC == P_BF16X2 ? 3 : wk == 1 || PREC == P_F32 ? 8 : PREC == P_FP8S ? 4 : 5;
+    const int per = nrhs == 1 ? 1
+                    : wk > 1  ? group_size(nrhs, cap, (int64_t)n_freq * groups, 1)
+                              : group_size(nrhs, cap, (int64_t)n_freq * ((groups + kFwdWarps - 1) / kFwdWarps), 2);
 #define BTT_FWD(NB) \
-    if (per <= NB) return fwd_multi<PREC, NB>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, per, st)
+    if (per <= NB) return fwd_multi<PREC, NB>(fhat, scales, n_freq, N_d, ldm, xh, xbs, dh, dbs, nrhs, per, wk, st)
+    BTT_FWD(1);
     BTT_FWD(2);
     BTT_FWD(3);
     if constexpr (PREC != P_BF16X2) {
@@ -512,11 +546,11 @@ template <int PREC, int... NB> static cudaError_t fwd_limits(std::integer_sequen
 // another thread's launch before the first has been made.
 cudaError_t prepare_gemv_multi()
 {
-    using Groups = std::integer_sequence<int, 2, 3, 4, 5, 6, 7, 8>;
+    using Groups = std::integer_sequence<int, 1, 2, 3, 4, 5, 6, 7, 8>;
     cudaError_t e = fwd_limits<P_F32>(Groups{});
     if (e == cudaSuccess) e = fwd_limits<P_F16S>(Groups{});
     if (e == cudaSuccess) e = fwd_limits<P_BF16>(Groups{});
-    if (e == cudaSuccess) e = fwd_limits<P_BF16X2>(std::integer_sequence<int, 2, 3>{});
+    if (e == cudaSuccess) e = fwd_limits<P_BF16X2>(std::integer_sequence<int, 1, 2, 3>{});
     if (e == cudaSuccess) e = fwd_limits<P_FP8S>(Groups{});
     return e;
 }

@@ -152,6 +152,9 @@ cudaError_t launch_gemv_adj(int prec, const void* fhat, const float* scales, int
 
 // Both for several vectors at once, FP32 formats (gemv_multi.cu).
 cudaError_t prepare_gemv_multi();
+// fwd_slices: warps that share a row of F there (1 or 8), by the operator's
+// shape; above 1 every F of the operator goes there, single vectors too.
+int fwd_slices(int prec, int n_freq, int N_d, int ldm);
 cudaError_t launch_gemv_fwd_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int ldm,
                                   const void* xh, int64_t xbs, void* dh, int64_t dbs, int nrhs, cudaStream_t st);
 cudaError_t launch_gemv_adj_multi(int prec, const void* fhat, const float* scales, int n_freq, int N_d, int N_m,
@@ -210,6 +213,8 @@ bool res_irfft(const float2* X, int64_t ldx, int64_t bsx, int ncols, float* y, i
                cudaError_t* err);
 bool res_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx, int ncols, float* y, int64_t ldy, int64_t bsy,
                     int nb, const FftGeom& g, const float2* tw, cudaStream_t st, float* const* yptr, cudaError_t* err);
+// Whether res_irfft and res_rfft are the faster middle step for ncols columns.
+bool res_mid(const FftGeom& g, int ncols);
 // True when 2 N_t has a fixed radix plan.
 bool static_plan(const FftGeom& g);
 // Its fixed-plan form; false for lengths without a fixed plan.

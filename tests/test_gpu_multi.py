@@ -54,3 +54,31 @@ def test_padding_columns_stay_zero():
         op.adjoint(bad)
         got = host(op.matvec(dev(m, torch.float32)))
     assert direct.rel_l2(got, direct.forward(F, m)) < TOL["f32"]
+
+
+FULL = [  # (N_t, N_d, N_m): grids of several waves, so that a batch of up to 8 stays one group
+    (600, 33, 70), (300, 33, 1100),
+]
+
+
+@pytest.mark.parametrize("shape", FULL)
+@pytest.mark.parametrize("prec", ["f32", "f16s", "bf16", "bf16x2", "fp8s"])
+def test_whole_groups(shape, prec):
+    """The kernels of 5 to 8 vectors (F* of FP8 up to 4; F of split pairs has its
+    own there): 601 x 2 tiles of rows are 4 waves of two CTAs per SM, where one pass
+    for all vectors costs 4 (n + 1) against 8 (n / 2 + 1) for two halves; F*
+    has 601 column tiles of 608 resident.  Every vector against the oracle's
+    algorithm on the same rounded Fhat (4e-6, as above)."""
+    N_t, N_d, N_m = shape
+    w = synth.Workload("groups", N_t, N_d, N_m, tau=N_t / 3, envelope=prec != "f32", seed=N_d * 7 + N_m)
+    F, m, d, _ = inputs(w, nrhs=8)
+    Fq = quantize.quantize(fft_method.setup(F), QFMT[prec])
+    fwd_q, adj_q = fft_method.forward(Fq, m), fft_method.adjoint(Fq, d)
+    with btt.Operator(torch.from_numpy(F).cuda(), precision=prec, max_nrhs=8, gemm="simt") as op:
+        for n in (2, 3, 4, 5, 6, 7, 8):
+            dm = host(op.matvec(dev(m[:n], torch.float32)))
+            md = host(op.adjoint(dev(d[:n], torch.float32)))
+            for j in range(n):
+                assert direct.rel_l2(dm[j], fwd_q[j]) < 4e-6
+                assert direct.rel_l2(md[j], adj_q[j]) < 4e-6
+        op.device_status()

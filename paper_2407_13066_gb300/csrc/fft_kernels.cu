@@ -286,8 +286,10 @@ __global__ void k_make_scales(const unsigned long long* __restrict__ maxbits, fl
 }
 
 // ---------------------------------------------------------------- launchers
-template <typename T> static size_t fft_smem(int L, int wc_log2) { return (size_t)(L << wc_log2) * sizeof(cplx_t<T>); }
-template <typename T> static size_t fft_smem(const FftGeom& g) { return fft_smem<T>(g.L, g.wc_log2); }
+template <typename T> static size_t fft_smem(const FftGeom& g)
+{
+    return (size_t)(g.L << g.wc_log2) * sizeof(cplx_t<T>);
+}
 
 static size_t create_smem(const FftGeom& g)
 {
@@ -313,9 +315,9 @@ bool runtime_fits(const FftGeom& g, bool fp64)
     return (fp64 ? fft_smem<double>(g) : fft_smem<float>(g)) <= (size_t)kFftSmemMax;
 }
 
-static dim3 col_grid(int ncols, int nb, int wc_log2)
+static dim3 col_grid(int ncols, int nb, const FftGeom& g)
 {
-    const int W = 2 << wc_log2;
+    const int W = 2 << g.wc_log2;
     return dim3((unsigned)((ncols + W - 1) / W), (unsigned)nb, 1);
 }
 
@@ -337,7 +339,6 @@ cudaError_t prepare_kernels()
 #define BTT_SET(k, b) \
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
     BTT_SET(k_rfft<float>, fmax_f);
-    BTT_SET(k_rfft<double>, fmax_d);
     BTT_SET(k_irfft<float>, fmax_f);
     BTT_SET((k_irfft<float, __nv_bfloat162>), fmax_f);
     BTT_SET(k_irfft<double>, fmax_d);
@@ -360,18 +361,6 @@ cudaError_t prepare_kernels()
     return e;
 }
 
-// Column pairs per CTA: the geometry's, but in FP64 as few as give two CTAs
-// per SM.  An SM has two FP64 lanes, so columns spread over more SMs are that
-// much faster whatever the rows' width: 64 steps and 32 columns ran on one SM
-// (26 us, its FP64 pipe 64% busy, the rest idle), now on 16 (5 us).
-template <typename T> static int tile_log2(int ncols, int nb, const FftGeom& g)
-{
-    int wc = g.wc_log2;
-    if (std::is_same<T, double>::value)
-        while (wc > 0 && (int64_t)nb * ((ncols + (2 << wc) - 1) / (2 << wc)) < 2 * 152) --wc;
-    return wc;
-}
-
 template <typename T>
 cudaError_t launch_rfft(const T* x, int64_t ldx, int64_t bsx, int ncols, cplx_t<T>* X,
                         int64_t ldo, int64_t bso, int nb, const FftGeom& g, const cplx_t<T>* tw,
@@ -385,14 +374,16 @@ cudaError_t launch_rfft(const T* x, int64_t ldx, int64_t bsx, int ncols, cplx_t<
         if (res_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e)) return e;
     }
     if constexpr (std::is_same<T, double>::value) {
-        cudaError_t e;
-        if (pf_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e)) return e;
+        // (one half needs 20 bytes per step: every length an FP64 operator may have)
+        cudaError_t e = cudaErrorNotSupported;
+        pf_rfft(x, ldx, bsx, ncols, X, ldo, bso, nb, g, tw, st, xptr, &e);
+        return e;
+    } else {
+        k_rfft<T><<<col_grid(ncols, nb, g), kFftThreads, fft_smem<T>(g), st>>>(
+            x, ldx, bsx, ncols, X, ldo, bso, g.N_t, g.plan, g.wc_log2, tw, g.pos, xptr);
+        count_launch();
+        return cudaGetLastError();
     }
-    const int wc = tile_log2<T>(ncols, nb, g);
-    k_rfft<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(
-        x, ldx, bsx, ncols, X, ldo, bso, g.N_t, g.plan, wc, tw, g.pos, xptr);
-    count_launch();
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -411,9 +402,8 @@ cudaError_t launch_irfft(const cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols
         cudaError_t e;
         if (pf_irfft(X, ldx, bsx, ncols, y, ldy, bsy, gam, nb, g, tw, st, yptr, &e)) return e;
     }
-    const int wc = tile_log2<T>(ncols, nb, g);
-    k_irfft<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(
-        X, ldx, bsx, ncols, y, ldy, bsy, gam, g.N_t, g.plan, wc, tw, g.pos, yptr);
+    k_irfft<T><<<col_grid(ncols, nb, g), kFftThreads, fft_smem<T>(g), st>>>(
+        X, ldx, bsx, ncols, y, ldy, bsy, gam, g.N_t, g.plan, g.wc_log2, tw, g.pos, yptr);
     count_launch();
     return cudaGetLastError();
 }
@@ -427,13 +417,13 @@ cudaError_t launch_irfft_bf16(const __nv_bfloat162* X, int64_t ldx, int64_t bsx,
     if (exchange_irfft_bf16(X, ldx, bsx, ncols, y, ldy, bsy, nb, g, tw, st, yptr, &e)) return e;
     if (static_irfft_bf16(X, ldx, bsx, ncols, y, ldy, bsy, nb, g, tw, st, yptr, &e)) return e;
     if (res_irfft_bf16(X, ldx, bsx, ncols, y, ldy, bsy, nb, g, tw, st, yptr, &e)) return e;
-    k_irfft<float, __nv_bfloat162><<<col_grid(ncols, nb, g.wc_log2), kFftThreads, fft_smem<float>(g), st>>>(
+    k_irfft<float, __nv_bfloat162><<<col_grid(ncols, nb, g), kFftThreads, fft_smem<float>(g), st>>>(
         X, ldx, bsx, ncols, y, ldy, bsy, nullptr, g.N_t, g.plan, g.wc_log2, tw, g.pos, yptr);
     count_launch();
     return cudaGetLastError();
 }
 
-int fft_col_blocks(int ncols, const FftGeom& g) { return (int)col_grid(ncols, 1, g.wc_log2).x; }
+int fft_col_blocks(int ncols, const FftGeom& g) { return (int)col_grid(ncols, 1, g).x; }
 
 template <typename T>
 cudaError_t launch_hess_mid(cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols, const T* gam,
@@ -460,9 +450,8 @@ cudaError_t launch_hess_mid(cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols, c
         cudaError_t e;
         if (pf_hess_mid(X, ldx, bsx, ncols, gam, nb, g, tw, st, &e)) return e;
     }
-    const int wc = tile_log2<T>(ncols, nb, g);
-    k_hess_mid<T><<<col_grid(ncols, nb, wc), kFftThreads, fft_smem<T>(g.L, wc), st>>>(
-        X, ldx, bsx, ncols, gam, g.N_t, g.plan, wc, tw, g.pos, part);
+    k_hess_mid<T><<<col_grid(ncols, nb, g), kFftThreads, fft_smem<T>(g), st>>>(
+        X, ldx, bsx, ncols, gam, g.N_t, g.plan, g.wc_log2, tw, g.pos, part);
     count_launch();
     return cudaGetLastError();
 }
@@ -496,7 +485,7 @@ cudaError_t launch_rfft_stack(const float* x, int64_t ldx, int64_t bsx, int ncol
         if (static_rfft_stack(x, ldx, bsx, ncols, xstack, ldm, mt_stride, nb, g, tw, st, lo_off, xptr, &e)) return e;
         if (res_rfft_stack(x, ldx, bsx, ncols, xstack, ldm, mt_stride, nb, g, tw, st, lo_off, xptr, &e)) return e;
     }
-    k_rfft_stack<<<col_grid(ncols, nb, g.wc_log2), kFftThreads, fft_smem<float>(g), st>>>(
+    k_rfft_stack<<<col_grid(ncols, nb, g), kFftThreads, fft_smem<float>(g), st>>>(
         x, ldx, bsx, ncols, static_cast<__nv_bfloat162*>(xstack), ldm, mt_stride, g.N_t, g.plan, g.wc_log2, tw,
         g.pos, xptr, lo_off);
     count_launch();

@@ -180,10 +180,7 @@ template <int R, int SG> __device__ __forceinline__ void rdft(cq* v)
     else if constexpr (R == 2 || R == 4 || R == 8) fq::dft<R, SG>(v);
     else if constexpr (R % 2 == 1 && R <= 7) rdft_odd<R, SG>(v);
     else if constexpr (R == 9) dft_square<3, SG>(v);
-    else if constexpr (R == 16) dft_square<4, SG>(v);
-    else if constexpr (R == 12) dft_pfa<4, 3, SG>(v);
-    else if constexpr (R == 15) dft_pfa<3, 5, SG>(v);
-    else dft_pfa<2, R / 2, SG>(v);
+    else dft_pfa<2, R / 2, SG>(v);   // 6, 10
 }
 
 // a twiddle for both lanes

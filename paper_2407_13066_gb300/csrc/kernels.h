@@ -92,7 +92,7 @@ cudaError_t launch_irfft(const cplx_t<T>* X, int64_t ldx, int64_t bsx, int ncols
                          const cplx_t<T>* tw, cudaStream_t st, T* const* yptr = nullptr);
 
 // In place: X <- rfft(pad(irfft(X)[:N_t] * g)) -- the step between the F and
-// F* passes of the Hessian (g = NULL means 1).  With part != NULL, block
+// F* passes of the Hessian (g = NULL means 1).  With part != NULL (FP32), block
 // (tile, b) also writes part[b * fft_col_blocks(ncols) + tile] = its share of
 // sum_t sum_col g (F m)^2, the Gamma^-1-weighted squared norm of vector b's
 // data (p.Hp for the CG solver).  scratch: NULL, or nb N_t ncols values the

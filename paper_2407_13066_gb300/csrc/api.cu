@@ -662,7 +662,7 @@ BTT_API btt_status btt_create(btt_op** out, const double* blocks, int N_t, int N
         }
     }
     double2* cscratch = nullptr;
-    if (const size_t csb = create_scratch_bytes(geom)) {
+    if (const size_t csb = create_scratch_bytes(geom, op->prec == P_F16S || op->prec == P_FP8S)) {
         cudaError_t e = cudaMalloc((void**)&cscratch, csb);
         if (e != cudaSuccess) {
             cudaGetLastError();

@@ -304,9 +304,9 @@ static int create_grid(int ntiles)
     return ntiles < nsm * 2 ? ntiles : nsm * 2;
 }
 
-size_t create_scratch_bytes(const FftGeom& g)
+size_t create_scratch_bytes(const FftGeom& g, bool scaled)
 {
-    if (create_smem(g) <= (size_t)kFftSmemMax) return 0;
+    if ((g.setup_tab && setup_fits(g.splan, scaled)) || create_smem(g) <= (size_t)kFftSmemMax) return 0;
     return (size_t)create_grid(0x7fffffff) * (size_t)(g.L << g.wc_log2) * sizeof(double2);
 }
 

@@ -51,8 +51,9 @@ bool make_fft_geom(int N_t, FftGeom* g);
 bool runtime_fits(const FftGeom& g, bool fp64);
 
 // Bytes of global scratch the setup transform needs when its FP64 buffer
-// does not fit in shared memory (0 when it does).
-size_t create_scratch_bytes(const FftGeom& g);
+// does not fit in shared memory (0 when it does).  scaled: a format whose
+// largest entries are found in a pass of their own.
+size_t create_scratch_bytes(const FftGeom& g, bool scaled);
 
 // Host: pos[k] for k < L, the digit-reversed position of frequency k.
 void digit_reversal(const FftGeom& g, int* pos);

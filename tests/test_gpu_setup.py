@@ -75,3 +75,11 @@ def test_scales_of_a_slice_that_holds_nan(shape, prec):
     with btt.Operator(F, precision=prec) as op:
         _, sc = op.copy_fhat()
     np.testing.assert_array_equal(sc, np.ones(N_t + 1))
+
+
+@pytest.mark.parametrize("shape", [(5250, 1, 4), (5400, 2, 3), (6000, 1, 3), (6400, 1, 2)])
+def test_stored_fhat_at_the_largest_tiles(shape):
+    """Up to 6456 steps the prime-factor tile fits (with the maxima of the scaled
+    formats up to 5282, their pass takes the mixed-radix kernel above), the
+    mixed-radix one to 5811 and in global scratch beyond."""
+    test_stored_fhat(shape)

@@ -1076,8 +1076,9 @@ const char* site_name(long long s)
 btt_status check_records()
 {
 #ifdef BTT_CHECK
-    cudaError_t (*units[])(long long*, bool) = {check_record_fft_static, check_record_gemv, check_record_gemv_multi, check_record_api,
-                                                check_record_fft_exchange, check_record_fft_residue};
+    cudaError_t (*units[])(long long*, bool) = {check_record_fft_static,   check_record_gemv,        check_record_gemv_multi,
+                                                check_record_api,          check_record_fft_exchange, check_record_fft_residue,
+                                                check_record_fft_setup};
     for (auto u : units) {
         long long rec[3] = {0, 0, 0};
         cudaError_t e = u(rec, true);

@@ -31,6 +31,15 @@ __device__ __forceinline__ double2 mul(double2 a, double2 w)
 {
     return make_double2(fma(-a.y, w.y, a.x * w.x), fma(a.y, w.x, a.x * w.y));
 }
+// tile element i of n
+__device__ __forceinline__ double2 get(const double2* buf, int i, int n)
+{
+    return BTT_IN(i, n, CK_FFT_SMEM) ? buf[i] : make_double2(0., 0.);
+}
+__device__ __forceinline__ void put(double2* buf, int i, int n, double2 v)
+{
+    if (BTT_IN(i, n, CK_FFT_SMEM)) buf[i] = v;
+}
 // a - i b and a + i b
 __device__ __forceinline__ double2 sub_i(double2 a, double2 b) { return make_double2(a.x + b.y, a.y - b.x); }
 __device__ __forceinline__ double2 add_i(double2 a, double2 b) { return make_double2(a.x - b.y, a.y + b.x); }
@@ -130,16 +139,17 @@ __device__ __forceinline__ void pass(double2* buf, int total, int S, int I, int 
         const int at = ((hi * R * SI + lo) << wcl) + c;
         double2 v[R];
 #pragma unroll
-        for (int i = 0; i < R; ++i) v[i] = buf[at + i * step];
+        for (int i = 0; i < R; ++i) v[i] = get(buf, at + i * step, total << wcl);
         dft_fwd<R>(v);
         if (S > 1) {
             const int n1 = lo / I;
             if (n1)
 #pragma unroll
-                for (int k = 1; k < R; ++k) v[k] = mul(v[k], __ldg(tw + n1 * k * tstep));
+                for (int k = 1; k < R; ++k)
+                    if (BTT_IN(n1 * k * tstep, S * R * tstep, CK_FFT_TABLE)) v[k] = mul(v[k], __ldg(tw + n1 * k * tstep));
         }
 #pragma unroll
-        for (int i = 0; i < R; ++i) buf[at + i * step] = v[i];
+        for (int i = 0; i < R; ++i) put(buf, at + i * step, total << wcl, v[i]);
     }
     __syncthreads();
 }
@@ -205,8 +215,8 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
                 if (n >= N) break;
                 const double2 w = __ldg(tw + n), h = make_double2(0.5 * z[u].x, 0.5 * z[u].y);
                 const int at = ((int)in[n] << wcl) + c;
-                buf[at] = h;
-                buf[(N << wcl) + at] = mul(h, w);
+                put(buf, at, N << wcl, h);
+                put(buf + (N << wcl), at, N << wcl, mul(h, w));
             }
         }
         __syncthreads();
@@ -225,7 +235,8 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
                 // w = 2 j + 1, partner N - 1 - j
                 const double2* half = buf + ((w & 1) ? (N << wcl) : 0);
                 const int jj = w & 1 ? N - 1 - j : (j ? N - j : 0);
-                const double2 z = half[((int)out[j] << wcl) + c], zc = half[((int)out[jj] << wcl) + c];
+                const double2 z = get(half, ((int)out[j] << wcl) + c, N << wcl);
+                const double2 zc = get(half, ((int)out[jj] << wcl) + c, N << wcl);
                 a = make_double2(z.x + zc.x, z.y - zc.y);
                 d = make_double2(z.y + zc.y, zc.x - z.x);
             }
@@ -241,6 +252,8 @@ k_create_pf(const double* __restrict__ blk, int64_t ldb, int ncols, int64_t col_
                 continue;
             }
             if (w > N || !one) continue;
+            if (!BTT_IN(o0, (int64_t)N_d * ldm, CK_FFT_STORE) || (both && !BTT_IN(o1, (int64_t)N_d * ldm, CK_FFT_STORE)))
+                continue;
             const int64_t row = (int64_t)w * N_d * ldm;
             if constexpr (PREC == P_F64) {
                 double2* f = reinterpret_cast<double2*>(fhat) + row;
@@ -322,8 +335,8 @@ __device__ __forceinline__ void store_half(const double2* half, int odd, int N, 
     const int c = threadIdx.x & ((1 << wcl) - 1);
     if (col >= ncols) return;
     for (int j = threadIdx.x >> wcl; 2 * j + odd <= N; j += NT >> wcl) {
-        const double2 z = half[((int)out[j] << wcl) + c];
-        const double2 zc = half[((int)out[odd ? N - 1 - j : (j ? N - j : 0)] << wcl) + c];
+        const double2 z = get(half, ((int)out[j] << wcl) + c, N << wcl);
+        const double2 zc = get(half, ((int)out[odd ? N - 1 - j : (j ? N - j : 0)] << wcl) + c, N << wcl);
         double2* o = X + (int64_t)(2 * j + odd) * ldx + col;
         o[0] = make_double2(z.x + zc.x, z.y - zc.y);
         if (col + 1 < ncols) o[1] = make_double2(z.y + zc.y, zc.x - z.x);
@@ -342,8 +355,8 @@ __device__ __forceinline__ void load_conj(double2* buf, int N, int wcl, const un
         if (w == 0 || w == N) a.y = b.y = 0.;   // real bins
         const int j = w >> 1, jj = w & 1 ? N - 1 - j : (j ? N - j : 0);
         double2* half = buf + (w & 1 ? (N << wcl) : 0);
-        half[((int)in[j] << wcl) + c] = make_double2(a.x - b.y, -(a.y + b.x));
-        if (jj != j) half[((int)in[jj] << wcl) + c] = make_double2(a.x + b.y, a.y - b.x);
+        put(half, ((int)in[j] << wcl) + c, N << wcl, make_double2(a.x - b.y, -(a.y + b.x)));
+        if (jj != j) put(half, ((int)in[jj] << wcl) + c, N << wcl, make_double2(a.x + b.y, a.y - b.x));
     }
 }
 
@@ -366,7 +379,7 @@ k_rfft_pf(const double* __restrict__ x, int64_t ldx, int64_t bsx, int ncols, dou
         double2 z = make_double2(0., 0.);
         if (col < ncols) z.x = 0.5 * xb[(int64_t)n * ldx];
         if (col + 1 < ncols) z.y = 0.5 * xb[(int64_t)n * ldx + 1];
-        buf[((int)t.in[n] << wcl) + c] = odd ? mul(z, __ldg(tw + n)) : z;
+        put(buf, ((int)t.in[n] << wcl) + c, N << wcl, odd ? mul(z, __ldg(tw + n)) : z);
     }
     __syncthreads();
     passes(buf, N, plan, wcl, tw);
@@ -394,7 +407,7 @@ k_irfft_pf(const double2* __restrict__ X, int64_t ldx, int64_t bsx, int ncols, d
     for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
         // conj(y) = (E + w_L^n O) / L
         const int at = ((int)t.out[n] << wcl) + c;
-        const double2 v = add(buf[at], mul(buf[(N << wcl) + at], __ldg(tw + n)));
+        const double2 v = add(get(buf, at, N << wcl), mul(get(buf + (N << wcl), at, N << wcl), __ldg(tw + n)));
         double p = v.x * inv, q = -v.y * inv;
         if (g) {
             p *= g[(int64_t)n * ncols + col];
@@ -424,24 +437,24 @@ k_mid_pf(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* __restri
     const double inv = 0.5 / (2. * N);   // the unpack's 1/2 with it
     for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
         const int at = ((int)t.out[n] << wcl) + c;
-        const double2 v = add(buf[at], mul(odd[at], __ldg(tw + n)));
+        const double2 v = add(get(buf, at, N << wcl), mul(get(odd, at, N << wcl), __ldg(tw + n)));
         double2 z = make_double2(v.x * inv, -v.y * inv);
         if (g) {
             if (col < ncols) z.x *= g[(int64_t)n * ncols + col];
             if (col + 1 < ncols) z.y *= g[(int64_t)n * ncols + col + 1];
         }
-        buf[at] = z;
+        put(buf, at, N << wcl, z);
     }
     __syncthreads();
     // back to the input positions through the odd half
     for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl)
-        odd[((int)t.in[n] << wcl) + c] = buf[((int)t.out[n] << wcl) + c];
+        put(odd, ((int)t.in[n] << wcl) + c, N << wcl, get(buf, ((int)t.out[n] << wcl) + c, N << wcl));
     __syncthreads();
     for (int n = threadIdx.x >> wcl; n < N; n += NT >> wcl) {
         const int at = ((int)t.in[n] << wcl) + c;
-        const double2 z = odd[at];
-        buf[at] = z;
-        odd[at] = mul(z, __ldg(tw + n));
+        const double2 z = get(odd, at, N << wcl);
+        put(buf, at, N << wcl, z);
+        put(odd, at, N << wcl, mul(z, __ldg(tw + n)));
     }
     __syncthreads();
     passes(buf, 2 * N, plan, wcl, tw);
@@ -627,3 +640,9 @@ bool setup_create(const double* blk, int64_t ldb, int ncols, int64_t col_base, i
 }
 
 }  // namespace btt
+
+#ifdef BTT_CHECK
+namespace btt {
+BTT_CHECK_TU(check_record_fft_setup)
+}  // namespace btt
+#endif

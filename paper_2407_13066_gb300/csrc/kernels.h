@@ -74,6 +74,7 @@ cudaError_t check_record_gemv_multi(long long* rec, bool clear);
 cudaError_t check_record_api(long long* rec, bool clear);
 cudaError_t check_record_fft_exchange(long long* rec, bool clear);
 cudaError_t check_record_fft_residue(long long* rec, bool clear);
+cudaError_t check_record_fft_setup(long long* rec, bool clear);
 #endif
 
 // ---- time transforms (fft_kernels.cu) ----

@@ -455,12 +455,14 @@ static cudaError_t fwd_dispatch(const void* fhat, const float* scales, int n_fre
 //   FP8   3 - 8, short      1.05     1.02     0.92       0.80       0.68      0.70
 //               long        0.7    0.46-0.63 0.39-0.89  0.57-0.76
 // (long: more than 12 blocks; BF16 3 - 4 on 305-608 groups 1.05 up to 40 blocks,
-// 0.94 and below beyond.)  Two vectors: mixed (BF16 0.9-1.4, FP32 0.8-1.4);
+// 0.94 and below beyond; 3 - 4 vectors of more than 16 rows under 4096 columns go
+// either way, 420 x 37 x 3001 in FP32 85 here and 92 there.)  Two vectors: mixed (BF16 0.9-1.4, FP32 0.8-1.4);
 // split pairs (16 more registers per row) 0.9-1.4, by whether groups of three
 // divide the batch.
 static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
 {
     if (nrhs < 3 || prec == P_BF16X2 || N_d > 32 * 65535) return false;   // (row tiles index grid.y)
+    if (nrhs <= 4 && ldm < 4096 && N_d > 16) return false;
     const int64_t groups = (int64_t)n_freq * ((N_d + 3) / 4);
     const bool few = nrhs <= 4, wide = ldm > 12 * (prec == P_F32 ? 64 : prec == P_FP8S ? 256 : 128);
     if (prec == P_F32) return groups > (few ? (wide ? 608 : 1216) : nrhs <= 12 ? 608 : 304);
@@ -472,16 +474,17 @@ static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
 // much as 18 columns per warp, so short rows gain (1000 x 100 x 1000 824 -> 731
 // us, 5000 x 10 x 200 183 -> 134) while enough CTAs keep the SMs busy.  Time on
 // two warps over eight, by CTAs and row length:
-//   CTAs             128   512    1000       1400       2000       4000       8192
-//   up to 152       ~1.0   1.5    1.6        1.7        2.0        2.1        2.7
-//   153 .. 304       0.9   0.9  1.0-1.15   1.0-1.25   1.0-1.26   1.1-2.3    1.1-2.5
-//   305 .. 608       0.7   0.8    0.9        0.9      0.9-1.26   1.0-1.6    1.0-1.7
-//   above 608        0.6   0.8    0.9        0.95       1.0        1.0        1.05
+//   CTAs            64      128      512    1000       1400       2000       4000      8192
+//   up to 152    0.95-1.0  0.9-1.3   1.5    1.6        1.7        2.0        2.1       2.7
+//   153 .. 304      0.7      0.9     0.9  1.0-1.15   1.0-1.25   1.0-1.26   1.1-2.3   1.1-2.5
+//   305 .. 608      0.7      0.7     0.8    0.9        0.9      0.9-1.26   1.0-1.6   1.0-1.7
+//   609 .. 4864     0.5      0.6     0.8    0.9        0.95       1.0        1.0       1.05
+//   above           0.45     0.55    0.8    0.9        0.93       0.97       1.0       1.0
 // The number of vectors has no part in it: a vector's sums keep their order.
 static bool f64_two_warps(int n_freq, int N_d, int ldm)
 {
     const int64_t ctas = (int64_t)n_freq * ((N_d + 3) / 4);
-    return ctas > 304 ? ldm <= 1400 : (ctas > 152 && ldm <= 512);
+    return ldm <= (ctas > 4864 ? 4096 : ctas > 304 ? 1400 : ctas > 152 ? 512 : 64);
 }
 
 cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int n_freq, int N_d,

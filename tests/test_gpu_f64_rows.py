@@ -1,5 +1,5 @@
 """FP64 F on two and on eight warps per CTA: either side of the lines between
-them (152 and 304 CTAs, rows of 512 and 1400 entries), against the oracle."""
+them (152 and 304 CTAs, rows of 64, 512 and 1400 entries), against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -11,9 +11,9 @@ from tests.test_gpu_parity import TOL
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = [  # (N_t, N_d, N_m)
-    (8, 7, 1347), (24, 1, 3958), (150, 3, 512), (150, 3, 520), (152, 4, 512), (152, 4, 513), (303, 2, 1400), (304, 2, 1400),
-    (304, 2, 1401), (75, 13, 1399), (1, 1, 1),
+SHAPES = [  # (N_t, N_d, N_m): 9 x 2, 25, 151, 161, 301, 316 and 76 x 4 CTAs
+    (8, 7, 1347), (24, 1, 3958), (150, 3, 64), (150, 3, 65), (150, 3, 512), (160, 4, 512), (160, 4, 513), (300, 2, 512),
+    (300, 2, 513), (315, 2, 1400), (315, 2, 1401), (75, 13, 1399), (1, 1, 1),
 ]
 
 

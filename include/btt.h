@@ -74,7 +74,9 @@ typedef enum {
 } btt_precision;
 
 /* Which units run the per-frequency products when several right-hand
- * sides are applied together. */
+ * sides are applied together.  On either kind of unit a vector's result has
+ * the same bits alone and in any batch; BTT_GEMM_AUTO chooses the units by the
+ * number of vectors. */
 typedef enum {
     BTT_GEMM_AUTO = 0,     /* tensor cores for BTT_BF16 / BTT_BF16_SPLIT and nrhs >= 16, else SIMT */
     BTT_GEMM_SIMT = 1,     /* always the streaming SIMT kernels */

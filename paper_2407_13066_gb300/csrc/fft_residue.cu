@@ -27,8 +27,9 @@
 // p is read at M - 1 - p.
 //
 // Against the one-CTA kernels of fft_kernels.cu, which this replaces wherever
-// a plan exists (us; 8 FP32 vectors, N_t N_m = 6.4 M, rows off 16-byte
-// boundaries; 614 MB, 91 us at the measured copy rate):
+// a plan exists but for few columns of long odd lengths (res_irfft, res_mid;
+// us; 8 FP32 vectors, N_t N_m = 6.4 M, rows off 16-byte boundaries; 614 MB, 91 us
+// at the measured copy rate):
 //   N_t               60    100    250    420   1125   1500   3000   9000
 //   input, before    616    530    449    486    692    669    954   1382
 //   input, here      189    203    236    246    338    336    373    494
@@ -52,7 +53,8 @@ using fq::mul;
 // Threads per CTA (threads_of); 24 warps per SM with 3, 2 or 1 CTAs.
 constexpr int kNT = 256, kNTLong = 384, kNTLongest = 768;
 constexpr int ctas_per_sm(int nt) { return nt == kNT ? 3 : nt == kNTLong ? 2 : 1; }
-// Radices up to 10 run in 80 registers, three CTAs per SM; up to 16 they take
+// Radices up to 10 run in 80 registers, three CTAs per SM (the inverse on
+// clusters of 8 spills 80-88 bytes of its 16 folded values); up to 16 they take
 // 128 (two CTAs), and the passes saved do not make up for the latency left
 // uncovered (N_t = 1500, 8 columns on 2 CTAs: 866 / 1147 us against 646 / 911).
 constexpr int kMaxRadix = 10;

@@ -88,6 +88,7 @@ constexpr int kFwdSmemMax = 128 * 1024;   // set by prepare_gemv_multi
 
 // Whether two blocks' raw units fit beside the accumulators in 128 registers,
 // and whether 80 registers (three CTAs of 8 warps per SM) hold the kernel.
+// (Most spill up to 36 bytes; FP16 with 8 vectors 156, once per block.)
 template <int PREC, int NB> constexpr bool fwd_pipelined()
 {
     return PREC == P_BF16X2 ? NB <= 3 : (NB <= 6 || PREC == P_F32);
@@ -522,8 +523,8 @@ static cudaError_t adj_groups(const void* fhat, const float* scales, int n_freq,
     if constexpr (PREC != P_FP8S) {
         BTT_ADJ(5);
         BTT_ADJ(6);
-        // (16-bit formats: 7 spills, which few rows do not make up for,
-        // 2000 x 7 x 3000 FP16 128 against 137 us)
+        // (16-bit formats: 7 spills 64 bytes, which few rows do not make up for:
+        // one shape, 2000 x 7 x 3000 FP16, 128 on 8 against 137 us)
         if (PREC == P_F32 || PREC == P_BF16X2 || N_d > 16) BTT_ADJ(7);
         BTT_ADJ(8);
     }

@@ -929,8 +929,8 @@ EncodeTiled encode_fn()
     return fn;
 }
 
-// shared memory the three-stage split forward may claim (its own barriers
-// and flags take the rest of the 227 KB)
+// shared memory the split forward (two to four stages) may claim (its own
+// barriers and flags take the rest of the 227 KB)
 constexpr int kSplitSmemMax = 226 * 1024;
 
 template <int NM, int STAGES> size_t fwd_smem(int ntile_rows)
@@ -965,10 +965,14 @@ TcPlan tc_plan(int n_freq, int N_d, int ldm, int max_nrhs, bool split)
     int maxs = p.ktiles / 8 > 0 ? p.ktiles / 8 : 1;
     int S = want < 1 ? 1 : (want > maxs ? maxs : want);
     {
-        // one CTA per SM (shared memory): among want .. 4 want splits take
-        // the one whose CTAs fill whole waves of nsm best, charging each
-        // split its partial tile (written, then read by the reduction)
-        // against the operand bytes of a tile
+        // among want .. 4 want splits take the one whose CTAs fill whole
+        // waves of nsm best, charging each split its partial tile (written,
+        // then read by the reduction) against the operand bytes of a tile.
+        // The costs are those of a batch of 49 to 64 vectors: 64 rows of
+        // spectra, a partial tile of 128 rows, one CTA per SM; smaller batches
+        // load and store fewer rows, and 97 to 160 rows of Fhat let two CTAs
+        // share an SM (launch_tc_fwd), but keep the operator's plan, so that a
+        // vector's sums do not depend on its batch
         const double ops = (double)(split ? 2 : 1) * (p.ntile_rows + 64) * p.K2 * 2;
         const double ptile = 2.0 * tc::kTileM * p.ntile_rows * 4;
         double best = 1e30;

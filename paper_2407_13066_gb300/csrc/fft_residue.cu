@@ -54,7 +54,7 @@ using fq::mul;
 constexpr int kNT = 256, kNTLong = 384, kNTLongest = 768;
 constexpr int ctas_per_sm(int nt) { return nt == kNT ? 3 : nt == kNTLong ? 2 : 1; }
 // Radices up to 10 run in 80 registers, three CTAs per SM (the inverse on
-// clusters of 8 spills 80-88 bytes of its 16 folded values); up to 16 they take
+// clusters of 8 spills 80-88 bytes); up to 16 they take
 // 128 (two CTAs), and the passes saved do not make up for the latency left
 // uncovered (N_t = 1500, 8 columns on 2 CTAs: 866 / 1147 us against 646 / 911).
 constexpr int kMaxRadix = 10;

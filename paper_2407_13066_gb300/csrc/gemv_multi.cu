@@ -88,7 +88,7 @@ constexpr int kFwdSmemMax = 128 * 1024;   // set by prepare_gemv_multi
 
 // Whether two blocks' raw units fit beside the accumulators in 128 registers,
 // and whether 80 registers (three CTAs of 8 warps per SM) hold the kernel.
-// (Most spill up to 36 bytes; FP16 with 8 vectors 156, once per block.)
+// (Most spill up to 36 bytes; FP16 with 8 vectors 156.)
 template <int PREC, int NB> constexpr bool fwd_pipelined()
 {
     return PREC == P_BF16X2 ? NB <= 3 : (NB <= 6 || PREC == P_F32);
@@ -472,10 +472,9 @@ static int group_size(int nrhs, int cap, int64_t ctas, int resident)
 {
     int best = 0;
     int64_t cost = 0;
-    for (int g = (nrhs + cap - 1) / cap; g <= nrhs; ++g) {
-        const int per = (nrhs + g - 1) / g;
-        if (best && per < 2) break;
-        const int64_t c = ((nrhs + per - 1) / per * ctas + 152 * resident - 1) / (152 * resident) * (per + 1);
+    for (int most = cap; most >= 2; --most) {   // (a batch may hold thousands of vectors)
+        const int g = (nrhs + most - 1) / most, per = (nrhs + g - 1) / g;
+        const int64_t c = (g * ctas + 152 * resident - 1) / (152 * resident) * (per + 1);
         if (!best || c < cost) best = per, cost = c;
     }
     return best;

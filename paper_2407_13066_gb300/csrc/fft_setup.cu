@@ -465,13 +465,18 @@ k_mid_pf(double2* X, int64_t ldx, int64_t bsx, int ncols, const double* __restri
 static size_t vec_smem(int N, int halves, int wcl) { return ((size_t)halves * N << wcl) * sizeof(double2) + (size_t)N * 4; }
 
 // Column pairs per CTA: up to 8, two CTAs per SM by shared memory, and as few
-// as give two CTAs per SM work (an SM has two FP64 lanes).
+// as give two CTAs per SM work (an SM has two FP64 lanes).  Where a tile is
+// small, its latency and not the FP64 rate, no more than the 304 CTAs that are
+// resident: a second wave took as long again (us, input / inverse / middle step
+// with it -> without: 9 steps, 468 columns x 2 12.3 / 14.4 / 23.6 -> 8.2 / 8.3 / 14.4; 64 steps
+// 16.4 / 18.5 / 31.1 -> 10.3 / 11.3 / 18.5).  Above 512 points a tile the second wave is the
+// better balance (360 steps, 700 columns x 2 47 / 47 / 86 with it, 62 / 59 / 108 without).
 static int vec_tile(int N, int halves, int ncols, int nb)
 {
     int w = 0;
     while (w < 3 && vec_smem(N, halves, w + 1) <= 113 * 1024) ++w;
-    const int64_t z = halves == 1 ? 2 : 1;
-    while (w > 0 && z * nb * ((ncols + (2 << w) - 1) / (2 << w)) < 2 * 152) --w;
+    auto ctas = [&](int v) { return (int64_t)(halves == 1 ? 2 : 1) * nb * ((ncols + (2 << v) - 1) / (2 << v)); };
+    while (w > 0 && ctas(w) < 2 * 152 && (ctas(w - 1) <= 2 * 152 || (N * halves << w) > 1024)) --w;
     return w;
 }
 

@@ -480,11 +480,13 @@ static bool fwd_multi_wins(int prec, int n_freq, int N_d, int ldm, int nrhs)
 //   305 .. 608      0.7      0.7     0.8    0.9        0.9      0.9-1.26   1.0-1.6   1.0-1.7
 //   609 .. 4864     0.5      0.6     0.8    0.9        0.95       1.0        1.0       1.05
 //   above           0.45     0.55    0.8    0.9        0.93       0.97       1.0       1.0
+// (one vector; with 16 from 1824 CTAs on 0.92 at 1700 to 2400 columns: 126 x 122 x
+// 1670 2831 us on two warps, 3101 on eight, with one vector 197 and 204).
 // The number of vectors has no part in it: a vector's sums keep their order.
 static bool f64_two_warps(int n_freq, int N_d, int ldm)
 {
     const int64_t ctas = (int64_t)n_freq * ((N_d + 3) / 4);
-    return ldm <= (ctas > 4864 ? 4096 : ctas > 304 ? 1400 : ctas > 152 ? 512 : 64);
+    return ldm <= (ctas > 4864 ? 4096 : ctas > 1824 ? 3000 : ctas > 304 ? 1400 : ctas > 152 ? 512 : 64);
 }
 
 cudaError_t launch_gemv_fwd(int prec, const void* fhat, const float* scales, int n_freq, int N_d,
